@@ -191,8 +191,8 @@ typedef struct {
                                    explores one configuration, 64..512, a
                                    multiple of 32; 0 = from the model's
                                    widest configuration level, and one warp
-                                   per configuration when that level's lanes
-                                   fit a warp (P <= 4 under GREEDY)          */
+                                   per configuration under GREEDY (P <= 10)
+                                   or when that level's lanes fit a warp     */
   uint32_t stage_chunk;         /* LEVEL engine: winners a warp stages in
                                    shared memory before it reserves frontier-
                                    log space and copies them out: 64 to 192,
@@ -256,11 +256,13 @@ typedef struct {
                             resolved); with CONFIG, table_slots is the
                             shared-memory table of one block and the log
                             holds one segment per configuration           */
-  uint32_t unit_threads; /* CONFIG: threads that explore one configuration:
-                            32 when one warp does (its widest level x lanes
-                            per state fits a warp and mc_options.
-                            unit_threads is 0), else the block's threads;
-                            0 with LEVEL                                  */
+  uint32_t unit_threads; /* CONFIG: threads that hold one configuration's
+                            widest level, lanes_per_state per state: 32 when
+                            it fits a warp and mc_options.unit_threads is 0,
+                            else the block's threads; 0 with LEVEL.  (With
+                            unit_threads 0 a warp explores GREEDY models of
+                            P <= 10 whatever this says: the subsets of the
+                            units that start together are its bitmap.)    */
   uint64_t unit_width;   /* bound on one configuration's widest level      */
 } mc_layout;
 

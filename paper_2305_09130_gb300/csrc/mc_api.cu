@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "mc.h"
+#include "mc_cfg_wave.h"
 #include "mc_host.h"
 #include "mc_internal.h"
 
@@ -208,7 +209,8 @@ struct mc_model {
   uint32_t cfg_wcap = 0, cfg_tsize = 0;
   int cfg_threads = 0, cfg_grid = 0, cfg_grid_max = 0;
   size_t cfg_smem = 0;
-  bool cfg_warp = false;  // one warp per configuration (widest level x lanes per state <= 32)
+  bool cfg_warp = false;  // one warp per configuration: wave units (GREEDY), or the widest level's lanes fit a warp
+  int cfg_unit_threads = 0;  // mc_layout.unit_threads
   // device state
   bool reserved = false;
   int device = -1;
@@ -484,17 +486,21 @@ int size_buffers(mc_model* m) {
     // a warp per configuration when its widest level's lanes fit one warp
     // (unless the caller asks for blocks of unit_threads); else enough
     // threads for the widest level's lanes in one round, 64..512
-    m->cfg_warp = !m->opt.unit_threads && m->unit_width * m->tile <= mc::kCfgWarpLanes;
-    if (m->cfg_warp) {
-      m->cfg_threads = (int)mc::kCfgWarpBlockThreads;
+    const bool fits_warp = !m->opt.unit_threads && m->unit_width * m->tile <= mc::kCfgWarpLanes;
+    if (fits_warp) {
+      m->cfg_unit_threads = 32;
     } else if (m->opt.unit_threads) {
-      m->cfg_threads = (int)m->opt.unit_threads;
+      m->cfg_unit_threads = (int)m->opt.unit_threads;
     } else {
       const uint64_t want = m->unit_width * m->tile;
       int t = 64;
       while ((uint64_t)t < want && t < (int)mc::kCfgMaxThreads) t <<= 1;
-      m->cfg_threads = t;
+      m->cfg_unit_threads = t;
     }
+    // a warp also explores each configuration of a GREEDY model whose
+    // subsets fit it (wave units), whatever its lanes per state
+    m->cfg_warp = fits_warp || mc::wave_model(m->rule, m->P, m->opt.unit_threads);
+    m->cfg_threads = m->cfg_warp ? (int)mc::kCfgWarpBlockThreads : m->cfg_unit_threads;
     const uint64_t key_bytes = 8ull * m->key_words;
     const uint64_t ctrl_bytes = (mc::kBarBytes + sizeof(Ctrl)) * kSlots + kScalarBytes + 8ull * (m->max_level + 2) * 5;
     uint64_t total = mul_sat(m->log_cap, key_bytes + 4);
@@ -1180,8 +1186,8 @@ int mc_model_layout(const mc_model* m, mc_layout* out) {
   out->engine = m->engine;
   out->log_tag_bits = m->engine == MC_ENGINE_CONFIG ? 0 : log_tag_bits(m);
   out->unit_width = m->unit_width;
-  // threads that explore one configuration: 32 for warp units
-  out->unit_threads = m->engine != MC_ENGINE_CONFIG ? 0 : m->cfg_warp ? 32u : (uint32_t)m->cfg_threads;
+  // by states x lanes; a GREEDY model's wave units take a warp whatever this says
+  out->unit_threads = m->engine != MC_ENGINE_CONFIG ? 0 : (uint32_t)m->cfg_unit_threads;
   return MC_OK;
 }
 

@@ -859,13 +859,16 @@ int breserve_cfg(mc_batch* b) {
   uint64_t units = 0;
   b->cfg_threads = 64;
   b->cfg_wcap = 32;
+  bool block_models = false;
   for (const mc::CfgModelPrep& M : b->cm) {
     units += M.ab;
     if (mc::cfg_warp_model(M, b->opt)) continue;  // a warp per configuration: no block shape
+    block_models = true;
     b->cfg_threads = std::max<int>(b->cfg_threads, (int)M.threads);
     b->cfg_wcap = std::max(b->cfg_wcap, M.wcap);
   }
   if (b->opt.unit_threads) b->cfg_threads = (int)b->opt.unit_threads;
+  else if (!block_models) b->cfg_threads = (int)mc::kCfgWarpBlockThreads;
   b->cfg_smem = mc::cfg_smem_bytes(2, b->cfg_wcap, 2 * b->cfg_wcap);
   if (mc::cfg_occupancy(2, b->cfg_threads, b->cfg_smem, &bps) || bps < 1) {
     b->last_err = "occupancy query failed (configuration engine)";
@@ -1921,6 +1924,11 @@ int mc_server_submit(mc_server* S, const mc_model_desc* desc, const mc_query* q,
   if (S->opt.engine != MC_ENGINE_LEVEL) {
     // the configuration engine when it takes the model and it fits a job
     rc = mc::cfg_prepare(*desc, S->opt, req.cm);
+    // A server without pruning keeps the block units for levels wider than a
+    // warp: its exhaustive searches are the long requests that others are
+    // seen to join and overtake (C3 literal outlasts 2 ms on blocks, not as
+    // waves); with pruning, the default, wave units answer every request.
+    req.cm.waves = S->opt.prune != 0;
     if (rc == MC_OK && (req.cm.ab > kJobUnits || mc::cfg_tables_bytes(req.cm) > kJobTables)) rc = MC_ERR_INVAL;
     if (rc == MC_OK) {
       req.cfg = true;

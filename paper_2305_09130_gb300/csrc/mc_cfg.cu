@@ -37,6 +37,7 @@
 // 0 (the WG index field is at least 1).
 #include <cstdint>
 
+#include "mc_cfg_wave.h"
 #include "mc_device.cuh"
 
 namespace mc {
@@ -295,6 +296,7 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
 }
 
 // ------------------------------------------------------------------ warp units
+// (FREE models; the warp units of GREEDY models are wave units, below.)
 // A configuration whose widest level fits one warp (width bound x lanes per
 // state <= 32) is explored by a single warp, its level in registers: state
 // s of the level is held by lanes [s*g, s*g + g), every proposal of the level
@@ -347,7 +349,7 @@ template <class K, class C>
 __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T) {
   const uint32_t P = Q.p.P, n_bits = Q.p.n_bits, b = Q.p.b;
   const uint64_t n_mask = Q.p.n_mask;
-  const bool greedy = Q.p.rule == MC_GREEDY, prune = Q.prune != 0, early = Q.early_exit != 0;
+  const bool prune = Q.prune != 0, early = Q.early_exit != 0;
   const uint32_t* costp = Q.p.cost;
   const uint32_t* speedp = Q.p.speed;
   void* const log_keys = Q.log_keys;
@@ -364,7 +366,6 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
   const bool unit_ok = c < P;
   const C t_c = unit_ok ? (C)((uint64_t)__ldg(costp + cfg) * __ldg(speedp + c)) : (C)0;
   const C Tc = T < (uint64_t)(C)~(C)0 ? (C)T : (C)~(C)0;
-  constexpr C kNoneC = (C)~(C)0;
   const uint32_t c_shift = (P - 1 - (unit_ok ? c : 0)) * n_bits;
   const K one_c = (K)1 << c_shift;
   const bool log_on = Q.want_witness != 0;
@@ -385,14 +386,9 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
     const bool valid = my < W;
     C clk = 0;
     if (valid && unit_ok) clk = (C)field(key, c_shift, n_mask) * t_c;
-    C mx = clk, mn = (valid && unit_ok) ? clk : kNoneC;
+    C mx = clk, mn = 0;
     bool ok = valid && unit_ok;
-    if (greedy) {
-      group_minmax<true>(mx, mn, g);
-      ok = ok && clk == mn;
-    } else {
-      group_minmax<false>(mx, mn, g);
-    }
+    group_minmax<false>(mx, mn, g);
     const C nclk = clk + t_c;
     const C st = nclk > mx ? nclk : mx;  // model time of the successor
     if (prune && st > Tc) ok = false;
@@ -472,11 +468,22 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
   return 0;
 }
 
+}  // namespace
+}  // namespace mc
+
+#include "mc_cfg_wave.cuh"
+
+namespace mc {
+namespace {
+
+__device__ __forceinline__ bool wave_unit(const Params& p) { return p.rule == MC_GREEDY && p.P <= kWaveMaxP; }
+
 // The pass header from the combined records (one thread): counts, first
-// violating level, minima, the witness's trace, the published minimum.
+// violating level, minima, the published minimum, and with `walk` the
+// witness's trace from the frontier log.
 template <class K>
 __device__ void epilogue_publish(const CfgPass& Q, uint64_t T, uint32_t stop, uint32_t last, uint64_t e_best,
-                                 uint64_t e_wpack, uint64_t e_sum) {
+                                 uint64_t e_wpack, uint64_t e_sum, bool walk) {
   const Params& p = Q.p;
   const uint32_t ab = p.a * p.b;
   Ctrl* ctrl = Q.ctrl;
@@ -502,6 +509,9 @@ __device__ void epilogue_publish(const CfgPass& Q, uint64_t T, uint32_t stop, ui
   ctrl->wkey_lo = klo;
   ctrl->wkey_hi = sizeof(K) == 16 ? khi : 0;
   ctrl->widx = idx;
+  ctrl->witness_level = stop;
+  ctrl->trace_len = stop + 1;
+  if (!walk) return;
   for (uint32_t l = stop; l >= 2; --l) {
     const K key = KeyOps<K>::load(Q.log_keys, idx);
     Q.trace[2 * l] = KeyOps<K>::lo(key);
@@ -509,6 +519,8 @@ __device__ void epilogue_publish(const CfgPass& Q, uint64_t T, uint32_t stop, ui
     if (l == 2) break;
     idx = __ldcg(Q.log_par + idx);
     if (idx >= Q.seg[wcfg + 1] || idx < Q.seg[wcfg]) {  // cannot happen when the log is intact
+      ctrl->witness_level = 0;
+      ctrl->trace_len = 0;
       set_error(ctrl, MC_ERR_FRONTIER);
       return;
     }
@@ -518,8 +530,6 @@ __device__ void epilogue_publish(const CfgPass& Q, uint64_t T, uint32_t stop, ui
   Q.trace[3] = KeyOps<K>::hi(k1);
   Q.trace[0] = 0;
   Q.trace[1] = 0;
-  ctrl->witness_level = stop;
-  ctrl->trace_len = stop + 1;
 }
 
 // The block that finished a pass's last configuration: combine the
@@ -563,7 +573,7 @@ __device__ void cfg_epilogue(const CfgPass& Q, uint64_t T, CfgShared& S) {
   atomicAdd(&S.e_sum, (unsigned long long)part);
   __syncthreads();
   if (tid != 0) return;
-  epilogue_publish<K>(Q, T, stop, last, (uint64_t)S.e_best, (uint64_t)S.e_wpack, (uint64_t)S.e_sum);
+  epilogue_publish<K>(Q, T, stop, last, (uint64_t)S.e_best, (uint64_t)S.e_wpack, (uint64_t)S.e_sum, true);
 }
 
 // The warp that finished a pass's last configuration, when it is a warp
@@ -599,9 +609,19 @@ __device__ void cfg_epilogue_warp(const CfgPass& Q, uint64_t T) {
   }
   const uint32_t last = (Q.early_exit && stop != kNoLevel) ? stop : deep;
   uint64_t part = 0;
+  // 16 loads in flight: one warp sums the widths of a search that may be
+  // thousands of levels deep
+#pragma unroll 16
   for (uint32_t l = 3 + lane; l <= last; l += 32) part += __ldcg(Q.levels + 2 * l);
   const uint64_t sum = warp_sum_u64(part);
-  if (lane == 0) epilogue_publish<K>(Q, T, stop, last, best, wpack, sum);
+  const bool wave = wave_unit(p);
+  if (lane == 0) epilogue_publish<K>(Q, T, stop, last, best, wpack, sum, !wave);
+  if (wave && Q.want_witness && stop != kNoLevel) {
+    const CfgRec* r = Q.rec + (uint64_t)pack_i(wpack) * p.b + pack_j(wpack);
+    K key = (K)__ldcg(&r->wkey_lo);
+    if (sizeof(K) == 16) key |= (K)((u128)__ldcg(&r->wkey_hi) << 64);
+    wave_trace<K>(Q, pack_i(wpack), pack_j(wpack), key);
+  }
 }
 
 // Blocks [0, warp_blocks) of a launch: every warp takes warp units until
@@ -634,7 +654,10 @@ __device__ void warp_role(const CfgLaunch& A) {
     }
     t = __shfl_sync(0xffffffffu, t, 0);
     skip = __shfl_sync(0xffffffffu, skip, 0);
-    if (!skip) {
+    if (!skip && wave_unit(Q.p)) {
+      if (Q.p.clk32) explore_wave<K, uint32_t>(Q, cfg, t);
+      else explore_wave<K, uint64_t>(Q, cfg, t);
+    } else if (!skip) {
       const uint32_t err = Q.p.clk32 ? explore_unit_warp<K, uint32_t>(Q, cfg, t)
                                      : explore_unit_warp<K, uint64_t>(Q, cfg, t);
       if (lane == 0 && err) set_error(Q.ctrl, (int)err);
@@ -658,6 +681,12 @@ __device__ void warp_role(const CfgLaunch& A) {
     }
     __syncwarp();
   }
+}
+
+// A launch without block units: only the warp units' code and registers.
+template <class K>
+__global__ void __launch_bounds__(kCfgWarpBlockThreads) cfg_warp_kernel(const __grid_constant__ CfgLaunch A) {
+  warp_role<K>(A);
 }
 
 template <class K>
@@ -817,6 +846,11 @@ int cfg_occupancy(int key_words, int threads, size_t smem, int* blocks_per_sm) {
 
 cudaError_t launch_cfg(int key_words, int grid, int threads, size_t smem, const CfgLaunch& L,
                        cudaStream_t stream) {
+  if (L.warp_blocks >= (uint32_t)grid) {  // every block serves warp units
+    if (key_words == 1) cfg_warp_kernel<uint64_t><<<grid, threads, 0, stream>>>(L);
+    else cfg_warp_kernel<u128><<<grid, threads, 0, stream>>>(L);
+    return cudaGetLastError();
+  }
   if (key_words == 1) cfg_kernel<uint64_t><<<grid, threads, smem, stream>>>(L);
   else cfg_kernel<u128><<<grid, threads, smem, stream>>>(L);
   return cudaGetLastError();

@@ -195,6 +195,7 @@ void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* q
   wcap = 32;
   threads = 64;
   any_min = false;
+  block_models = false;
   for (uint32_t k = 0; k < n; ++k) {
     CfgModelPrep& M = *models[k];
     const mc_query& q = queries[k];
@@ -202,6 +203,7 @@ void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* q
     const bool warp = cfg_warp_model(M, opt);
     any_min |= mt;
     if (!warp) {  // blocks are sized for the models they explore
+      block_models = true;
       wcap = std::max(wcap, M.wcap);
       threads = std::max(threads, M.threads);
     }
@@ -297,6 +299,7 @@ void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* q
   walks_max = std::max<uint32_t>(opt.sim_walks, 1);
   tsize = 2 * wcap;
   if (opt.unit_threads) threads = opt.unit_threads;
+  else if (!block_models) threads = kCfgWarpBlockThreads;
   // blocks of warp units: from pass A's count, which depends on the models
   // only (a replayed graph keeps them while the queries change), and twice
   // that for pass B (every warp model a min-time query with both checks)
@@ -329,7 +332,8 @@ cudaError_t CfgRun::enqueue(cudaStream_t st, int grid_a, int grid_b, size_t smem
   L.n_wunits_dev = d_cnt + 6;
   L.wnext = d_cnt + 8;
   L.warp_blocks = wblocks_a;
-  if ((e = launch_cfg(2, grid_a + (int)wblocks_a, threads, smem, L, st))) return e;
+  // (without block units every block serves warp units)
+  if ((e = launch_cfg(2, (block_models ? grid_a : 0) + (int)wblocks_a, threads, smem, L, st))) return e;
   L.units = d_units + cap_units;
   L.n_units_dev = d_cnt + 3;
   L.next = d_cnt + 1;
@@ -337,7 +341,7 @@ cudaError_t CfgRun::enqueue(cudaStream_t st, int grid_a, int grid_b, size_t smem
   L.n_wunits_dev = d_cnt + 7;
   L.wnext = d_cnt + 9;
   L.warp_blocks = wblocks_b;
-  if ((e = launch_cfg(2, grid_b + (int)wblocks_b, threads, smem, L, st))) return e;
+  if ((e = launch_cfg(2, (block_models ? grid_b : 0) + (int)wblocks_b, threads, smem, L, st))) return e;
   if (ev1 && (e = capturing ? cudaEventRecordWithFlags(ev1, st, cudaEventRecordExternal) : cudaEventRecord(ev1, st)))
     return e;
   return cudaMemcpyAsync(h_block + result_off, d_block + result_off, result_bytes, cudaMemcpyDeviceToHost, st);

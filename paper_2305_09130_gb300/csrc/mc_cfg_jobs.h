@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "mc.h"
+#include "mc_cfg_wave.h"
 #include "mc_internal.h"
 
 namespace mc {
@@ -17,6 +18,7 @@ struct CfgModelPrep {
   Params p;                    // table pointers into the region once placed
   uint32_t group = 1, ab = 0, L2 = 0, threads = 64, wcap = 32;
   uint64_t unit_width = 0, unit_log = 0, region = 0;
+  bool waves = true;             // wave units allowed (mc_cfg_wave.h)
   std::vector<uint32_t> params;  // N, cost, speed
   std::vector<uint64_t> seg;     // [ab + 1]
   std::vector<uint32_t> order;   // configurations, deepest first
@@ -33,10 +35,12 @@ struct CfgModelPrep {
 // Validate the description and lay the model out (host only).  Errors: as
 // mc_model_create, INVAL when the configuration engine cannot take it.
 int cfg_prepare(const mc_model_desc& d, const mc_options& o, CfgModelPrep& M);
-// One warp per configuration: the widest level's lanes fit a warp and the
-// options leave the block's threads to the library.
+// One warp per configuration: the options leave the block's threads to the
+// library, and the model takes wave units or its widest level's lanes fit a
+// warp.
 inline bool cfg_warp_model(const CfgModelPrep& M, const mc_options& o) {
-  return !o.unit_threads && M.unit_width * M.group <= kCfgWarpLanes;
+  return (M.waves && wave_model(M.p.rule, M.p.P, o.unit_threads)) ||
+         (!o.unit_threads && M.unit_width * M.group <= kCfgWarpLanes);
 }
 // Point the model at its region (M.region bytes, 256-byte aligned); the
 // caller uploads M.params and M.seg to M.base and M.d_seg.
@@ -68,6 +72,7 @@ struct CfgRun {
   // the same unit regions, from their ends backwards; blocks serving them
   uint64_t n_wunits_a = 0, n_wunits_b = 0;
   uint32_t wblocks_a = 0, wblocks_b = 0;
+  bool block_models = false;  // some model takes block units
   bool refine = true, any_min = false;
 
   uint64_t tables_cap = 0, tables_used = 0;     // model tables carried by the upload
