@@ -39,6 +39,7 @@
 
 #include "mc_cfg_wave.h"
 #include "mc_device.cuh"
+#include "mc_walk.cuh"
 
 namespace mc {
 namespace {
@@ -790,16 +791,19 @@ __global__ void cfg_clear_kernel(const CfgClear* clears, const uint32_t* n_dev) 
 }
 
 // T_ini of every min-time model of a run: walk w of model k is random run
-// number w of its seed (as mc_simulate), the least terminal time wins.
+// number w of its seed (as mc_simulate), the least terminal time wins.  A
+// warp per run.
 __global__ void cfg_sim_kernel(const CfgSim* sims, const uint32_t* n_dev, uint32_t walks_max) {
   const uint32_t n = *n_dev;
   const uint64_t total = (uint64_t)n * walks_max;
-  for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
-       x += (uint64_t)gridDim.x * blockDim.x) {
+  for (uint64_t x = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < total;
+       x += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
     const uint32_t k = (uint32_t)(x / walks_max), w = (uint32_t)(x % walks_max);
     const CfgSim& s = sims[k];
     if (w >= s.walks) continue;
-    atomicMin(reinterpret_cast<unsigned long long*>(s.tini), (unsigned long long)simulate_walk(s.p, s.seed, w));
+    const uint64_t t = warp_walk_time(s.p, s.seed, w);
+    if ((threadIdx.x & 31u) == 0)
+      atomicMin(reinterpret_cast<unsigned long long*>(s.tini), (unsigned long long)t);
   }
 }
 
@@ -815,9 +819,8 @@ cudaError_t launch_cfg_clear(const CfgClear* clears, const uint32_t* n_dev, uint
 cudaError_t launch_cfg_sim(const CfgSim* sims, const uint32_t* n_dev, uint32_t n_max, uint32_t walks_max,
                            cudaStream_t stream) {
   if (n_max == 0 || walks_max == 0) return cudaSuccess;
-  const uint64_t total = (uint64_t)n_max * walks_max;
-  int grid = (int)((total + 127) / 128);
-  if (grid > 4096) grid = 4096;
+  const uint64_t blocks = ((uint64_t)n_max * walks_max + 3) / 4;  // 4 warps each
+  const int grid = (int)(blocks < 4096 ? blocks : 4096);
   cfg_sim_kernel<<<grid, 128, 0, stream>>>(sims, n_dev, walks_max);
   return cudaGetLastError();
 }

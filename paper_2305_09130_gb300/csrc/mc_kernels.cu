@@ -4,6 +4,7 @@
 #include <cstdint>
 
 #include "mc_explore.cuh"
+#include "mc_walk.cuh"
 
 namespace mc {
 namespace {
@@ -11,32 +12,30 @@ namespace {
 using namespace mc::dev;
 
 // ------------------------------------------------------------------ simulation (T_ini)
-// One random run per thread (Section 4, Step 3: a simulation gives T_ini).
+// One random run per warp (Section 4, Step 3: a simulation gives T_ini).
 __global__ void simulate_kernel(const Params p, uint64_t seed, uint32_t walks, uint64_t* t_out) {
-  const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t w = gtid; w < walks; w += nthreads)
-    atomicMin(reinterpret_cast<unsigned long long*>(t_out),
-              (unsigned long long)simulate_walk(p, seed, w));
+  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  uint64_t least = kNone;
+  for (uint64_t w = warp; w < walks; w += nwarps) {
+    const uint64_t t = warp_walk_time(p, seed, w);
+    least = t < least ? t : least;
+  }
+  if ((threadIdx.x & 31u) == 0 && least != kNone)
+    atomicMin(reinterpret_cast<unsigned long long*>(t_out), (unsigned long long)least);
 }
 
 // ------------------------------------------------------------------ swarm (Section 5)
 // Walks w0 .. w0 + walks - 1, each cut as soon as a clock passes `bound`;
 // the least (time, walk) over the runs that end at or below the bound goes to
 // *best as (time << 24) | (w - w0).
+template <class C, int PT>
 __global__ void swarm_kernel(const Params p, uint64_t seed, uint64_t w0, uint32_t walks,
                              uint64_t bound, unsigned long long* best) {
   const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
-  unsigned long long mine = kNone;
-  for (uint64_t k = gtid; k < walks; k += nthreads) {
-    const uint64_t t = walk_time(p, seed, w0 + k, bound);
-    if (t != kNone) {
-      const unsigned long long v = ((unsigned long long)t << 24) | k;
-      mine = v < mine ? v : mine;
-    }
-  }
-  mine = warp_min(mine);
+  const unsigned long long mine =
+      warp_min(swarm_runs<C, PT>(p, seed, w0, gtid, nthreads, walks, bound));
   if ((threadIdx.x & 31u) == 0 && mine != kNone) atomicMin(best, mine);
 }
 
@@ -135,7 +134,14 @@ cudaError_t launch_explore(int key_words, int tile, int rule, int scheme, int gr
 
 cudaError_t launch_swarm(const Params& p, uint64_t seed, uint64_t w0, uint32_t walks, uint64_t bound,
                          unsigned long long* best, int grid, cudaStream_t stream) {
-  swarm_kernel<<<grid, 256, 0, stream>>>(p, seed, w0, walks, bound, best);
+  // the clocks in registers, 32 bits wide where every clock of the model fits
+#define MC_SWARM(PT)                                                                             \
+  (p.clk32 ? swarm_kernel<uint32_t, PT><<<grid, 256, 0, stream>>>(p, seed, w0, walks, bound, best) \
+           : swarm_kernel<uint64_t, PT><<<grid, 256, 0, stream>>>(p, seed, w0, walks, bound, best))
+  if (p.P <= 4) MC_SWARM(4);
+  else if (p.P <= 8) MC_SWARM(8);
+  else MC_SWARM(16);
+#undef MC_SWARM
   return cudaGetLastError();
 }
 
@@ -148,8 +154,8 @@ cudaError_t launch_replay_walk(const Params& p, uint64_t seed, uint64_t w, int k
 cudaError_t launch_simulate(const Params& p, uint64_t seed, uint32_t walks, uint64_t* t_out,
                             cudaStream_t stream) {
   const int threads = 128;
-  int grid = (int)((walks + threads - 1) / threads);
-  if (grid > 1024) grid = 1024;
+  const uint64_t blocks = ((uint64_t)walks * 32 + threads - 1) / threads;  // a warp per walk
+  const int grid = (int)(blocks < 4096 ? blocks : 4096);
   simulate_kernel<<<grid, threads, 0, stream>>>(p, seed, walks, t_out);
   return cudaGetLastError();
 }
