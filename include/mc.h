@@ -81,9 +81,14 @@ typedef enum {
  * 32-byte bucket into shared memory first; CAS_FIRST starts with the
  * compare-and-swap.  The results are identical, only the speed differs. */
 typedef enum {
-  MC_PROBE_AUTO = 0,     /* SPLIT with 64-bit keys, CAS_FIRST with 128-bit
-                            (the fastest on C2 at G=80, whose table stays in
-                            L2, and on C3 at G=36, whose probes go to DRAM) */
+  MC_PROBE_AUTO = 0,     /* FREE models, unless table_log2 or max_probes is
+                            set: no insert -- a state proposes a unit only
+                            when no later unit has started, so each state
+                            is generated once and no visited set is kept.
+                            Else SPLIT with 64-bit keys, CAS_FIRST with
+                            128-bit (the fastest on C2 at G=80, whose table
+                            stays in L2, and on C3 at G=36, whose probes go
+                            to DRAM)                                        */
   MC_PROBE_SPLIT = 1,    /* pick the slot from the fetched bucket, issue the
                             CAS of every proposal of the round, then resolve
                             (a lost slot or a full bucket falls back to the
@@ -239,13 +244,15 @@ typedef struct {
   uint32_t P, n_bits, ts_bits, wg_bits, ts_shift, wg_shift;
   uint32_t max_level;    /* deepest BFS level: max N_ij + 2                */
   uint32_t n_shift[16];
-  uint64_t table_slots;  /* visited-set slots                              */
+  uint64_t table_slots;  /* visited-set slots (what a named insert takes;
+                            AUTO on a FREE model keeps no visited set, and
+                            device_bytes leaves it out)                    */
   uint64_t log_capacity; /* frontier-log entries                           */
   uint64_t max_width;    /* bound on one level's width                     */
   uint64_t state_bound;  /* bound on all reachable states (saturates)      */
   uint64_t device_bytes; /* device memory the model needs                  */
-  uint32_t probe_scheme; /* the insert its explorations use (mc_probe_scheme,
-                            AUTO resolved)                                 */
+  uint32_t probe_scheme; /* the insert of its visited set (mc_probe_scheme,
+                            AUTO resolved by key width)                    */
   uint32_t log_tag_bits; /* bits per 64-bit word of a frontier-log entry
                             that tag it with its pass, so a block can arrive
                             at a level's barrier before writing its last

@@ -17,6 +17,7 @@
 #include "mc_cfg_wave.h"
 #include "mc_host.h"
 #include "mc_internal.h"
+#include "mc_tree.h"
 
 using mc::Ctrl;
 using mc::ExploreArgs;
@@ -206,6 +207,7 @@ struct mc_model {
   std::vector<uint64_t> seg;       // [a*b + 1] segment starts
   std::vector<uint32_t> order;     // [a*b] configurations, deepest first
   uint32_t engine = MC_ENGINE_LEVEL;
+  bool ordered = false;  // level engine: ordered expansion (no visited set)
   uint32_t cfg_wcap = 0, cfg_tsize = 0;
   int cfg_threads = 0, cfg_grid = 0, cfg_grid_max = 0;
   size_t cfg_smem = 0;
@@ -469,10 +471,21 @@ int resolve_scheme(uint32_t scheme, uint32_t key_words) {
   return (int)scheme;
 }
 
+// The level engine expands FREE models in order (mc_tree.cu) unless the
+// options name an insert or size the visited set: each state is generated
+// once, so there is nothing to look up.  Measured min-time queries against the
+// AUTO inserts: C3 at G=36 (1.07e9 states, bound by random access to the
+// visited set) 266.9 -> 7.2 ms, C2 at G=80 (10.4M states) 1.16 -> 0.39 ms.
+bool resolve_ordered(const mc_model* m) {
+  return m->rule == MC_FREE && m->opt.probe_scheme == MC_PROBE_AUTO && m->opt.table_log2 == 0 &&
+         m->opt.max_probes == 0;
+}
+
 // sizes of the frontier log and the visited set
 int size_buffers(mc_model* m) {
   if (resolve_tile(m)) return MC_ERR_INVAL;
   m->engine = resolve_engine(m);
+  m->ordered = m->engine == MC_ENGINE_LEVEL && resolve_ordered(m);
   if (m->engine == MC_ENGINE_CONFIG) {
     if (!cfg_eligible(m)) return MC_ERR_INVAL;
     // a segment of the log per configuration, shared-memory tables per block
@@ -532,7 +545,7 @@ int size_buffers(mc_model* m) {
   m->table_slots = slots;
   const uint64_t key_bytes = 8ull * m->key_words;
   const uint64_t ctrl_bytes = (mc::kBarBytes + sizeof(Ctrl)) * kSlots + kScalarBytes + 8ull * (m->max_level + 2) * 5;
-  uint64_t total = mul_sat(slots, key_bytes);
+  uint64_t total = m->ordered ? 0 : mul_sat(slots, key_bytes);  // (ordered expansion keeps no visited set)
   total = add_sat(total, mul_sat(m->log_cap, key_bytes + 4));
   total = add_sat(total, ctrl_bytes + 4ull * (2ull * m->a * m->b + m->P));
   m->device_bytes = total;
@@ -587,9 +600,13 @@ int reserve(mc_model* m) {
       m->last_err = "device lacks cooperative launch";
       return MC_ERR_CUDA;
     }
-    m->threads = m->opt.threads_per_block ? (int)m->opt.threads_per_block : (int)mc::kThreads;
+    m->threads = m->opt.threads_per_block ? (int)m->opt.threads_per_block
+                 : m->ordered             ? mc::kTreeThreads
+                                          : (int)mc::kThreads;
     m->scheme = resolve_scheme(m->opt.probe_scheme, m->key_words);
-    if (mc::explore_kernel_occupancy(m->key_words, m->tile, m->rule, m->scheme, m->threads, &bps) || bps < 1) {
+    if ((m->ordered ? mc::tree_occupancy(m->key_words, m->used_bits, m->threads, &bps)
+                    : mc::explore_kernel_occupancy(m->key_words, m->tile, m->rule, m->scheme, m->threads, &bps)) ||
+        bps < 1) {
       m->last_err = "occupancy query failed";
       cudaGetLastError();
       return MC_ERR_CUDA;
@@ -617,7 +634,8 @@ int reserve(mc_model* m) {
   const uint64_t key_bytes = 8ull * m->key_words;
   const size_t np = 2ull * m->a * m->b + m->P;
   m->d_params = (uint32_t*)dev_alloc(m, np * 4);
-  if (!cfg) m->d_table = dev_alloc(m, m->table_slots * key_bytes);
+  const bool table = !cfg && !m->ordered;
+  if (table) m->d_table = dev_alloc(m, m->table_slots * key_bytes);
   m->d_log_keys = dev_alloc(m, m->log_cap * key_bytes);
   m->d_log_par = (uint32_t*)dev_alloc(m, m->log_cap * 4);
   const size_t L2 = m->max_level + 2;
@@ -632,7 +650,7 @@ int reserve(mc_model* m) {
     m->d_pair_pass = (mc::CfgPass*)dev_alloc(m, 8 * sizeof(mc::CfgPass));
     m->d_pair_units = (uint64_t*)dev_alloc(m, 8 * 3 * ab);
   }
-  if (!m->d_params || (!cfg && !m->d_table) || !m->d_log_keys || !m->d_log_par || !m->d_ctrl_block ||
+  if (!m->d_params || (table && !m->d_table) || !m->d_log_keys || !m->d_log_par || !m->d_ctrl_block ||
       (cfg && (!m->d_seg || !m->d_rec || !m->d_order || !m->d_cfg_levels || !m->d_pair_pass ||
                !m->d_pair_units))) {
     release(m);
@@ -653,6 +671,7 @@ int reserve(mc_model* m) {
   // tagged frontier log for 64-bit keys with 8 or more spare top bits: the
   // log starts cleared, so no entry of freed memory carries a tag
   m->tag_bits = cfg ? 0 : log_tag_bits(m);  // the configuration engine's log is read only after its pass
+  if (m->ordered) m->tag_bits = mc::tree_tag_bits((int)m->key_words, m->used_bits, m->tag_bits);
   m->tag = 0;
   if (m->tag_bits) MC_CUDA(m, cudaMemsetAsync(m->d_log_keys, 0, m->log_cap * key_bytes, m->stream));
 
@@ -888,7 +907,9 @@ int enqueue_pass(mc_model* m, uint64_t T, const uint64_t* T_src, int64_t delta, 
     const int rc_ = timed_launch(m);
     if (rc_) return rc_;
   }
-  MC_CUDA(m, mc::launch_explore(m->key_words, m->tile, m->rule, m->scheme, m->grid, m->threads, A, m->stream));
+  if (m->ordered) MC_CUDA(m, mc::launch_tree(m->key_words, m->used_bits, m->grid, m->threads, A, m->stream));
+  else
+    MC_CUDA(m, mc::launch_explore(m->key_words, m->tile, m->rule, m->scheme, m->grid, m->threads, A, m->stream));
   m->stats.explore_launches += 1;
   return MC_OK;
 }
