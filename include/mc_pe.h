@@ -85,7 +85,7 @@ typedef struct {
   uint32_t wg_shift, ts_shift, level_shift, max_level;
   uint32_t unit_shift[8];
   uint64_t max_steps;    /* longest program in steps                        */
-  uint64_t table_slots;  /* visited-set slots                               */
+  uint64_t table_slots;  /* visited-set slots, where one is kept            */
   uint64_t log_capacity; /* frontier-log entries                            */
   uint64_t device_bytes; /* device memory of the current buffers            */
 } mc_pe_layout;
@@ -96,8 +96,11 @@ typedef struct {
  * the frontier log start at table_log2 / log_capacity when given, else at
  * 2^20 slots and 2^22 entries, and grow fourfold (up to half the device's
  * free memory, and the visited set up to 2^31 slots) whenever a query ends
- * in TABLE_FULL or FRONTIER, which then reruns; max_probes 0 means 64 bucket
- * probes.  Errors: INVAL, OVERFLOW (also table_log2 > 31). */
+ * in TABLE_FULL or FRONTIER, which then reruns.  The visited set is only kept
+ * when table_log2 or max_probes is set: else a state's events since the last
+ * tick are taken in one order (by unit, then by PE), which generates every
+ * state once (lanes_per_state belongs to the pass with a visited set; there
+ * max_probes 0 means 64 bucket probes).  Errors: INVAL, OVERFLOW (also table_log2 > 31). */
 int mc_pe_model_create(const mc_pe_model_desc* desc, const mc_options* opt, mc_pe_model** out);
 void mc_pe_model_destroy(mc_pe_model* m);
 int mc_pe_set_stream(mc_pe_model* m, void* stream);

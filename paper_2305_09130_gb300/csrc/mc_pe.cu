@@ -34,6 +34,7 @@ using namespace mc::dev;
 constexpr uint32_t kPeMaxUnits = 8;
 constexpr uint32_t kPeMaxPes = 8;
 constexpr uint32_t kBarrierBit = 1u << 16;  // step info: barrier flag | participating PEs
+constexpr uint32_t kEnteredBit = 1u << 17;  // step info: entered by a dispatch or past a barrier, not by a tick
 // successors per lane a tile of `tile` lanes can propose: one for a whole
 // warp, two for half a warp, three for smaller tiles
 __host__ __device__ constexpr uint32_t slots_for(uint32_t tile) { return tile >= 32 ? 1 : tile == 16 ? 2 : 3; }
@@ -48,7 +49,8 @@ struct PeParams {
   const uint32_t* tau;     // [a*b] ticks of one program
   const uint32_t* nsteps;  // [a*b] steps of one program
   const uint32_t* soff;    // [a*b] first step of each program
-  const uint2* step;       // [steps] {barrier bit | pes, ticks before the step}
+  const uint2* step;       // [steps] {entered bit | barrier bit | pes, ticks before the step}
+  const uint4* cfg4;       // [a*b] {N, tau, steps | ends with a barrier << 31, first step}
 };
 
 struct PeArgs {
@@ -74,7 +76,8 @@ struct PeArgs {
   uint32_t* bar;
   uint64_t timeout_ns;
   uint32_t slots;    // successors per lane: ceil(lanes / TILE) <= slots_for(TILE)
-  uint32_t pad;
+  uint32_t tag_bits; // ordered expansion: the log's tag (mc_explore.cuh), 0 bits: untagged
+  uint64_t tag;
 };
 
 struct Unit {
@@ -569,6 +572,8 @@ uint32_t bits_for(uint64_t x) {
 }  // namespace
 }  // namespace mc
 
+#include "mc_pe_ordered.cuh"
+
 // ------------------------------------------------------------------ host side
 struct mc_pe_model {
   uint32_t a = 0, b = 0, P = 0, M = 0;
@@ -579,6 +584,10 @@ struct mc_pe_model {
   mc::PeParams params{};
   uint64_t table_slots = 0, log_cap = 0;
   uint32_t max_probes = 64;
+  // ordered expansion (no visited set) unless the options size the visited
+  // set; its log tag
+  bool ordered = false;
+  uint32_t tag_bits = 0, tag = 0;
   // device state
   int device = -1, grid = 0, threads = 0;
   cudaStream_t stream = nullptr;
@@ -657,8 +666,8 @@ void* pe_alloc(mc_pe_model* m, size_t bytes) {
 
 uint64_t pe_device_bytes(const mc_pe_model* m) {
   const uint64_t L2 = m->lay.max_level + 2;
-  return m->table_slots * 16 + m->log_cap * 20 + 256 + mc::kBarBytes + 40 * L2 + 64 +
-         4ull * (4 * (uint64_t)m->a * m->b) + 8ull * m->steps.size();
+  return (m->ordered ? 0 : m->table_slots * 16) + m->log_cap * 20 + 256 + mc::kBarBytes + 40 * L2 + 64 +
+         4ull * (8 * (uint64_t)m->a * m->b) + 8ull * m->steps.size();
 }
 
 int pe_reserve(mc_pe_model* m) {
@@ -673,10 +682,13 @@ int pe_reserve(mc_pe_model* m) {
     m->last_err = "device lacks cooperative launch";
     return MC_ERR_CUDA;
   }
-  m->threads = m->opt.threads_per_block ? (int)m->opt.threads_per_block : (int)mc::kThreads;
+  m->threads = m->opt.threads_per_block ? (int)m->opt.threads_per_block
+               : m->ordered             ? mc::kPeThreads
+                                        : (int)mc::kThreads;
   int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, mc::pe_pick(m->lay.tile), m->threads, 0) !=
-          cudaSuccess ||
+  const void* kernel = m->ordered ? mc::pe_ordered_pick(m->params) : mc::pe_pick(m->lay.tile);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, m->threads,
+                                                    m->ordered ? sizeof(mc::PeSoloShared) : 0) != cudaSuccess ||
       bps < 1) {
     cudaGetLastError();
     m->last_err = "occupancy query failed";
@@ -687,13 +699,13 @@ int pe_reserve(mc_pe_model* m) {
 
   const size_t ab = (size_t)m->a * m->b;
   const size_t L2 = m->lay.max_level + 2;
-  uint32_t* d_cfg = (uint32_t*)pe_alloc(m, 4 * 4 * ab);
+  uint32_t* d_cfg = (uint32_t*)pe_alloc(m, 8 * 4 * ab);
   uint2* d_steps = (uint2*)pe_alloc(m, 8 * m->steps.size());
-  m->d_table = pe_alloc(m, m->table_slots * 16);
+  if (!m->ordered) m->d_table = pe_alloc(m, m->table_slots * 16);
   m->d_log_keys = pe_alloc(m, m->log_cap * 16);
   m->d_log_par = (uint32_t*)pe_alloc(m, m->log_cap * 4);
   uint8_t* q = (uint8_t*)pe_alloc(m, 256 + mc::kBarBytes + 40 * L2 + 64);
-  if (!d_cfg || !d_steps || !m->d_table || !m->d_log_keys || !m->d_log_par || !q) {
+  if (!d_cfg || !d_steps || (!m->ordered && !m->d_table) || !m->d_log_keys || !m->d_log_par || !q) {
     pe_release(m);
     return MC_ERR_NOMEM;
   }
@@ -719,11 +731,19 @@ int pe_reserve(mc_pe_model* m) {
   m->h_trace = (uint64_t*)(m->h_block + o_trace);
   if (m->opt.timing && !m->ev[0])
     for (cudaEvent_t& e : m->ev) PE_CUDA(m, cudaEventCreate(&e));
-  std::vector<uint32_t> cfg(4 * ab);
+  std::vector<uint32_t> cfg(8 * ab);  // four arrays, then the same as one record per configuration
   std::copy(m->N.begin(), m->N.end(), cfg.begin());
   std::copy(m->tau.begin(), m->tau.end(), cfg.begin() + ab);
   std::copy(m->nsteps.begin(), m->nsteps.end(), cfg.begin() + 2 * ab);
   std::copy(m->soff.begin(), m->soff.end(), cfg.begin() + 3 * ab);
+  for (size_t k = 0; k < ab; ++k) {
+    const bool barrier_end = m->steps[m->soff[k] + m->nsteps[k] - 1].x & mc::kBarrierBit;
+    uint32_t* q4 = &cfg[4 * ab + 4 * k];
+    q4[0] = m->N[k];
+    q4[1] = m->tau[k];
+    q4[2] = m->nsteps[k] | (barrier_end ? 1u << 31 : 0u);
+    q4[3] = m->soff[k];
+  }
   // pageable sources: these copies complete before the calls return
   PE_CUDA(m, cudaMemcpy(d_cfg, cfg.data(), 4 * cfg.size(), cudaMemcpyHostToDevice));
   PE_CUDA(m, cudaMemcpy(d_steps, m->steps.data(), 8 * m->steps.size(), cudaMemcpyHostToDevice));
@@ -734,6 +754,12 @@ int pe_reserve(mc_pe_model* m) {
   p.nsteps = d_cfg + 2 * ab;
   p.soff = d_cfg + 3 * ab;
   p.step = d_steps;
+  p.cfg4 = (const uint4*)(d_cfg + 4 * ab);
+  // tagged log: cleared, so no entry of freed memory carries a tag
+  const uint32_t spare = (128 - m->lay.used_bits) / 2;
+  m->tag_bits = m->ordered && !m->opt.no_log_tags && spare >= 8 ? std::min<uint32_t>(spare, 16) : 0;
+  m->tag = 0;
+  if (m->tag_bits) PE_CUDA(m, cudaMemsetAsync(m->d_log_keys, 0, m->log_cap * 16, m->stream));
   m->lay.table_slots = m->table_slots;
   m->lay.log_capacity = m->log_cap;
   m->lay.device_bytes = pe_device_bytes(m);
@@ -772,9 +798,18 @@ int pe_enqueue(mc_pe_model* m, uint64_t T, const uint64_t* T_src, int64_t delta,
   if (m->opt.timing && !m->ev[0])
     for (cudaEvent_t& e : m->ev) PE_CUDA(m, cudaEventCreate(&e));
   if (m->opt.timing) PE_CUDA(m, cudaEventRecord(m->ev[2 * slot], m->stream));
+  if (m->tag_bits) {  // a new tag per pass; the log is cleared when the tags wrap
+    if (++m->tag >= (1u << m->tag_bits)) {
+      PE_CUDA(m, cudaMemsetAsync(m->d_log_keys, 0, m->log_cap * 16, m->stream));
+      m->tag = 1;
+    }
+    A.tag_bits = m->tag_bits;
+    A.tag = m->tag;
+  }
   void* args[] = {&A};
-  PE_CUDA(m, cudaLaunchCooperativeKernel(mc::pe_pick(m->lay.tile), dim3(m->grid), dim3(m->threads), args, 0,
-                                         m->stream));
+  PE_CUDA(m, cudaLaunchCooperativeKernel(m->ordered ? mc::pe_ordered_pick(m->params) : mc::pe_pick(m->lay.tile),
+                                         dim3(m->grid), dim3(m->threads), args,
+                                         m->ordered ? sizeof(mc::PeSoloShared) : 0, m->stream));
   if (m->opt.timing) {
     PE_CUDA(m, cudaEventRecord(m->ev[2 * slot + 1], m->stream));
     m->ev_pending[slot] = true;
@@ -910,16 +945,21 @@ int mc_pe_model_create(const mc_pe_model_desc* d, const mc_options* opt, mc_pe_m
     M = std::max(M, nwe);
     uint64_t ticks = 0, marks = 0, barriers = 0, S = 0;
     m->soff.push_back((uint32_t)m->steps.size());
+    // the step about to be added is the program's first or follows a barrier
+    auto entered = [m]() -> uint32_t {
+      return m->steps.size() == m->soff.back() || (m->steps.back().x & mc::kBarrierBit) ? mc::kEnteredBit : 0u;
+    };
     for (uint32_t s = d->prog_off[k]; s < d->prog_off[k + 1]; ++s) {
       const uint32_t t = d->seg_ticks[s], pe = d->seg_pes[s];
       if (pe == 0 || pe > nwe || t > 65535) return fail(MC_ERR_INVAL);
       if (t == 0) {
-        m->steps.push_back(make_uint2(mc::kBarrierBit | pe, (uint32_t)ticks));
+        m->steps.push_back(make_uint2(mc::kBarrierBit | pe | entered(), (uint32_t)ticks));
         marks += pe;
         barriers += 1;
         S += 1;
       } else {
-        for (uint32_t x = 0; x < t; ++x) m->steps.push_back(make_uint2(pe, (uint32_t)(ticks + x)));
+        for (uint32_t x = 0; x < t; ++x)
+          m->steps.push_back(make_uint2(pe | (x == 0 ? entered() : 0u), (uint32_t)(ticks + x)));
         ticks += t;
         marks += (uint64_t)t * pe;
         S += t;
@@ -989,6 +1029,7 @@ int mc_pe_model_create(const mc_pe_model_desc* d, const mc_options* opt, mc_pe_m
   const uint64_t n_init = 1 + (uint64_t)m->a + ab;
   m->log_cap = std::max<uint64_t>(o.log_capacity ? o.log_capacity : (1ull << 22), n_init);
   m->max_probes = o.max_probes ? o.max_probes : 64;
+  m->ordered = o.table_log2 == 0 && o.max_probes == 0;
   L.table_slots = m->table_slots;
   L.log_capacity = m->log_cap;
   L.device_bytes = pe_device_bytes(m);

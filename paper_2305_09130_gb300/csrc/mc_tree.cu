@@ -269,7 +269,10 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
 #pragma unroll
     for (int r = 0; r < kTreeKeys; ++r)
       if (r < (int)R && base + r * blockDim.x < Wl) raw[r] = LogIO<K>::load(src, base + r * blockDim.x, lpol);
-    for (bool more = true; more;) {
+    // (a block without a state of the level only arrives)
+    bool more = base - tid < Wl;
+    if (!more && G.tag_bits && tid == 0) (void)level_arrive_reserve(lvl_next, &s_flags, stop_mask, 0);
+    while (more) {
       more = base - tid + stride < Wl;  // (uniform: the block's tiles end together)
       A key[kTreeKeys];
       // which units start: field f of the key (at f * n_bits) is unit P-1-f.
@@ -330,13 +333,11 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
       if (lane == 0) s_cnt[warp] = wcnt;
       if (!more && best != kNone) atomicMin(&s_best, (unsigned long long)best);
       __syncthreads();
+      // every warp sums the counts below its own, and all of them
+      const uint32_t wc = lane < nw ? s_cnt[lane] : 0u;
+      const uint32_t total = __reduce_add_sync(0xffffffffu, wc);
+      const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wc : 0u);
       if (tid == 0) {
-        uint32_t total = 0;
-        for (uint32_t w = 0; w < nw; ++w) {
-          const uint32_t c = s_cnt[w];
-          s_cnt[w] = total;
-          total += c;
-        }
         if (!more && s_best != kNone) {
           atomicMin(reinterpret_cast<unsigned long long*>(lvl_next + 1), s_best);
           s_best = kNone;
@@ -349,7 +350,7 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
       }
       __syncthreads();
       if (wcnt) {
-        const uint64_t at0 = offN + s_base + s_cnt[warp];
+        const uint64_t at0 = offN + s_base + before;
         if (at0 + wcnt <= G.log_cap) {
           K* const dst = reinterpret_cast<K*>(G.log_keys) + at0;
           uint32_t* const par = G.log_par + at0;
