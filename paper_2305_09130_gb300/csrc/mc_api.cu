@@ -185,9 +185,33 @@ uint64_t binom_sat(uint64_t n, uint64_t k) {
 
 uint64_t add_sat(uint64_t a, uint64_t b) { return a > UINT64_MAX - b ? UINT64_MAX : a + b; }
 uint64_t mul_sat(uint64_t a, uint64_t b) {
-  if (a == 0 || b == 0) return 0;
-  return a > UINT64_MAX / b ? UINT64_MAX : a * b;
+  uint64_t r;
+  return __builtin_mul_overflow(a, b, &r) ? UINT64_MAX : r;
 }
+
+// The closed-form bound of one configuration's level k: C(k + P - 1, P - 1)
+// states of sum(n) = k, under GREEDY at most C(P, floor(P/2)).  It grows with
+// k until it reaches that cap or saturates.
+struct LevelBound {
+  uint32_t P;
+  uint64_t cap;
+  uint32_t k = 0;
+  uint64_t free_width = 1;
+  LevelBound(uint32_t units, uint64_t c) : P(units), cap(c) {}
+  uint64_t width() const { return std::min(free_width, cap); }
+  bool final() const { return free_width >= cap; }  // (cap is UINT64_MAX under FREE)
+  void next() {
+    ++k;
+    uint64_t x;
+    if (final()) return;
+    if (!__builtin_mul_overflow(free_width, (uint64_t)k + P - 1, &x)) {
+      free_width = x / k;
+    } else {
+      const unsigned __int128 nx = (unsigned __int128)free_width * (k + P - 1) / k;
+      free_width = nx > (unsigned __int128)UINT64_MAX ? UINT64_MAX : (uint64_t)nx;
+    }
+  }
+};
 
 }  // namespace
 
@@ -1088,46 +1112,53 @@ int mc_model_create(const mc_model_desc* d, const mc_options* opt, mc_model** ou
   //   GREEDY: at most C(P, floor(P/2)) per configuration and level, since
   //           after k dispatches only the units tied at the next start time
   //           can differ.
-  const uint64_t greedy_cap = binom_sat(m->P, m->P / 2);
-  // configurations with N_ij >= k, for every k (suffix sums of a histogram)
-  std::vector<uint64_t> at_least(n_max + 2, 0);
-  for (size_t k = 0; k < ab; ++k) at_least[m->N[k]] += 1;
-  for (int64_t k = (int64_t)n_max - 1; k >= 0; --k) at_least[k] += at_least[k + 1];
-  uint64_t total = add_sat(1 + (uint64_t)m->a, ab);
-  uint64_t widest = 0;
-  uint64_t per_free = 1;  // C(k+P-1, P-1), updated incrementally (saturating)
-  for (uint32_t k = 1; k <= n_max; ++k) {
-    if (per_free != UINT64_MAX) {
-      const unsigned __int128 nx = (unsigned __int128)per_free * (k + m->P - 1) / k;
-      per_free = nx > (unsigned __int128)UINT64_MAX ? UINT64_MAX : (uint64_t)nx;
-    }
-    uint64_t per = per_free;
-    if (m->rule == MC_GREEDY) per = std::min(per, greedy_cap);
-    const uint64_t w = mul_sat(per, at_least[k]);
-    widest = std::max(widest, w);
-    total = add_sat(total, w);
+  // The levels up to the one from which the bound stays the same are taken
+  // one by one, the deeper ones together (thousands of levels under GREEDY,
+  // where the bound is constant after a few).
+  const uint64_t cap = m->rule == MC_GREEDY ? binom_sat(m->P, m->P / 2) : UINT64_MAX;
+  LevelBound w(m->P, cap);
+  std::vector<uint64_t> width{w.width()}, upto{w.width()};  // the bound of level k, and of levels 0..k
+  while (w.k < n_max && !w.final()) {
+    w.next();
+    width.push_back(w.width());
+    upto.push_back(add_sat(upto.back(), w.width()));
   }
+  const uint32_t k_top = w.k;
+  const uint64_t w_top = w.width();  // every level from k_top on
+  // configurations with N_ij >= k for k <= k_top (suffix sums of a histogram)
+  std::vector<uint64_t> at_least(k_top + 2, 0);
+  uint64_t deeper = 0, beyond = 0;  // levels beyond k_top, summed; configurations that reach one
+  for (size_t k = 0; k < ab; ++k) {
+    at_least[std::min(m->N[k], k_top)] += 1;
+    if (m->N[k] > k_top) {
+      deeper += m->N[k] - k_top;
+      beyond += 1;
+    }
+  }
+  for (int64_t k = (int64_t)k_top - 1; k >= 0; --k) at_least[k] += at_least[k + 1];
+  uint64_t total = add_sat(1 + (uint64_t)m->a, ab);
+  uint64_t widest = mul_sat(w_top, beyond);
+  for (uint32_t k = 1; k <= k_top; ++k) {
+    const uint64_t level = mul_sat(width[k], at_least[k]);
+    widest = std::max(widest, level);
+    total = add_sat(total, level);
+  }
+  total = add_sat(total, mul_sat(w_top, deeper));
   m->max_width = widest;
   m->state_bound = total;
   // the configuration engine's bounds: the widest level of one
-  // configuration is w(n_max) (w grows with k), and configuration c's
-  // states number at most sum_{k <= N_c} w(k); its frontier-log segment
-  // has that size.  Configurations are taken deepest first.
+  // configuration is its bound at n_max (it grows with k), and configuration
+  // c's states number at most the sum of the bounds of levels 0..N_c; its
+  // frontier-log segment has that size.  Configurations are taken deepest
+  // first.
   {
-    std::vector<uint64_t> upto(n_max + 1);  // sum_{k' <= k} w(k')
-    uint64_t pf = 1, acc = 0;
-    for (uint32_t k = 0; k <= n_max; ++k) {
-      if (k > 0 && pf != UINT64_MAX) {
-        const unsigned __int128 nx = (unsigned __int128)pf * (k + m->P - 1) / k;
-        pf = nx > (unsigned __int128)UINT64_MAX ? UINT64_MAX : (uint64_t)nx;
-      }
-      const uint64_t w = m->rule == MC_GREEDY ? std::min(pf, greedy_cap) : pf;
-      acc = add_sat(acc, w);
-      upto[k] = acc;
-      if (k == n_max) m->unit_width = w;
-    }
+    m->unit_width = w_top;
     m->seg.assign(ab + 1, 0);
-    for (size_t k = 0; k < ab; ++k) m->seg[k + 1] = add_sat(m->seg[k], upto[m->N[k]]);
+    for (size_t k = 0; k < ab; ++k) {
+      const uint32_t n = m->N[k];
+      const uint64_t own = n <= k_top ? upto[n] : add_sat(upto[k_top], mul_sat(w_top, n - k_top));
+      m->seg[k + 1] = add_sat(m->seg[k], own);
+    }
     m->unit_log = m->seg[ab];
     m->order.resize(ab);
     for (size_t k = 0; k < ab; ++k) m->order[k] = (uint32_t)k;

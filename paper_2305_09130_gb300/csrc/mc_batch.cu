@@ -900,6 +900,9 @@ int breserve_cfg(mc_batch* b) {
     b->stats.h2d_bytes += 4 * M.params.size() + 8 * M.seg.size();
   }
   MCB_CUDA(b, cudaStreamSynchronize(b->stream));
+  std::vector<mc::CfgModelPrep*> ms(b->n);
+  for (uint32_t i = 0; i < b->n; ++i) ms[i] = &b->cm[i];
+  b->run.order_units(ms, b->opt);
   b->trace_len.assign(b->n, 0);
   b->reserved = true;
   return MC_OK;
@@ -1661,6 +1664,7 @@ bool admit_jobs(mc_server* S) {
     if (j.reqs.empty()) break;  // the front request waits for pool room
     std::vector<mc::CfgModelPrep*> ms(j.reqs.size());
     for (size_t k = 0; k < j.reqs.size(); ++k) ms[k] = &j.reqs[k].cm;
+    j.run.order_units(ms, S->opt);
     j.run.prepare(ms, j.qs.data(), S->opt);
     size_t smem = 0;
     const int grid = job_grid(S, j.run.threads, j.run.wcap, &smem);

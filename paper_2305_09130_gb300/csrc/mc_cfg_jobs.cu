@@ -185,13 +185,22 @@ void CfgRun::layout(uint32_t n_max, uint64_t units_max, uint8_t* dev, uint8_t* h
   h_tables = host + o_tab;
 }
 
+void CfgRun::order_units(const std::vector<CfgModelPrep*>& models, const mc_options& opt) {
+  order.clear();
+  for (uint32_t k = 0; k < (uint32_t)models.size(); ++k) {
+    const CfgModelPrep& M = *models[k];
+    const uint32_t warp = cfg_warp_model(M, opt);
+    for (uint32_t c : M.order) order.push_back({M.params[c], k, c, warp});  // (params begin with N)
+  }
+  std::stable_sort(order.begin(), order.end(), [](const Unit& x, const Unit& y) { return x.n > y.n; });
+}
+
 void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* queries, const mc_options& opt) {
   const uint32_t n = (uint32_t)models.size();
   n_models = n;
   refine = opt.refine != 0;
   std::memset(h_cnt, 0, 256);
   uint32_t n_sim = 0;
-  std::vector<std::pair<uint32_t, uint64_t>> ua, ub, wa, wb;  // (work-groups, unit) for sorting
   wcap = 32;
   threads = 64;
   any_min = false;
@@ -257,36 +266,24 @@ void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* q
     C.ctrl = d_ctrl + 3ull * k;
     C.n_ctrl = 3;
     C.scal = scal;
-    const uint32_t* N = M.params.data();
-    auto& la = warp ? wa : ua;
-    auto& lb = warp ? wb : ub;
-    for (uint32_t c : M.order) {
-      la.push_back({N[c], ((uint64_t)(3 * k) << 32) | c});
-      if (mt) {
-        if (refine) lb.push_back({N[c], ((uint64_t)(3 * k + 1) << 32) | c});
-        lb.push_back({N[c], ((uint64_t)(3 * k + 2) << 32) | c});
-      }
-    }
   }
-  // deepest configurations first within each launch
-  auto deeper = [](const std::pair<uint32_t, uint64_t>& x, const std::pair<uint32_t, uint64_t>& y) {
-    return x.first > y.first;
-  };
-  std::stable_sort(ua.begin(), ua.end(), deeper);
-  std::stable_sort(ub.begin(), ub.end(), deeper);
-  std::stable_sort(wa.begin(), wa.end(), deeper);
-  std::stable_sort(wb.begin(), wb.end(), deeper);
-  n_units_a = ua.size();
-  n_units_b = ub.size();
-  n_wunits_a = wa.size();
-  n_wunits_b = wb.size();
   // pass A's region [0, cap), pass B's [cap, 3 cap): block units from the
   // start, warp units from the end backwards (a model's configurations are
-  // in one list or the other, so the two never meet)
-  for (uint64_t x = 0; x < ua.size(); ++x) h_units[x] = ua[x].second;
-  for (uint64_t x = 0; x < ub.size(); ++x) h_units[cap_units + x] = ub[x].second;
-  for (uint64_t x = 0; x < wa.size(); ++x) h_units[cap_units - 1 - x] = wa[x].second;
-  for (uint64_t x = 0; x < wb.size(); ++x) h_units[3 * cap_units - 1 - x] = wb[x].second;
+  // in one list or the other, so the two never meet); deepest configurations
+  // first within each launch
+  uint64_t ua = 0, ub = 0, wa = 0, wb = 0;
+  for (const Unit& u : order) {
+    const uint64_t unit = ((uint64_t)(3 * u.model) << 32) | u.cfg, pass = 1ull << 32;
+    const bool mt = queries[u.model].kind == MC_QUERY_MIN_TIME;
+    auto b = [&](uint64_t x) { h_units[u.warp ? 3 * cap_units - 1 - wb++ : cap_units + ub++] = x; };
+    h_units[u.warp ? cap_units - 1 - wa++ : ua++] = unit;
+    if (mt && refine) b(unit + pass);
+    if (mt) b(unit + 2 * pass);
+  }
+  n_units_a = ua;
+  n_units_b = ub;
+  n_wunits_a = wa;
+  n_wunits_b = wb;
   // counters: [0] next unit of pass A, [1] of pass B, [2] units of A,
   // [3] units of B, [4] models to clear, [5] min-time models to simulate,
   // [6] warp units of A, [7] of B, [8] next warp unit of A, [9] of B

@@ -75,6 +75,13 @@ struct CfgRun {
   bool block_models = false;  // some model takes block units
   bool refine = true, any_min = false;
 
+  // the (model, configuration) units, deepest first: made by order_units,
+  // kept while the models stay the same (a batch's runs)
+  struct Unit {
+    uint32_t n, model, cfg, warp;
+  };
+  std::vector<Unit> order;
+
   uint64_t tables_cap = 0, tables_used = 0;     // model tables carried by the upload
   uint8_t *d_tables = nullptr, *h_tables = nullptr;
 
@@ -83,7 +90,9 @@ struct CfgRun {
   // Copy M's tables and segment starts into the upload and point M at them
   // (false when they do not fit); reset with tables_used = 0 per run.
   bool place_tables(CfgModelPrep& M);
-  // Fill the pinned descriptors for queries[k] on *models[k].
+  void order_units(const std::vector<CfgModelPrep*>& models, const mc_options& opt);
+  // Fill the pinned descriptors for queries[k] on *models[k] (the models of
+  // the last order_units).
   void prepare(const std::vector<CfgModelPrep*>& models, const mc_query* queries, const mc_options& opt);
   // Upload, clear, simulate, both pass launches, read back (events around
   // the pass launches if given).

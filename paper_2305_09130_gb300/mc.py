@@ -8,9 +8,11 @@ library is missing or no CUDA device is usable, the calls raise.
 """
 from __future__ import annotations
 
+import array
 import atexit
 import ctypes as C
 import os
+import struct
 import threading
 import weakref
 from typing import Optional
@@ -316,7 +318,11 @@ class Model:
 
 
 def _u32(xs):
-    return (C.c_uint32 * len(xs))(*[int(x) for x in xs])
+    n = len(xs)
+    try:  # a list of ints: one copy (the ctypes array keeps the buffer alive)
+        return (C.c_uint32 * n).from_buffer(array.array("I", xs))
+    except (TypeError, OverflowError, ValueError):  # other numbers, or no elements
+        return (C.c_uint32 * n)(*[int(x) for x in xs])
 
 
 def mc_model_create(spec, options: Optional[McOptions] = None, allocator: Optional[str] = "torch",
@@ -599,11 +605,13 @@ def mc_batch_run(batch: Batch, queries) -> list:
     n = len(batch.specs)
     q = (McQuery * n)()
     for k, (kind, T) in enumerate(queries):
-        q[k] = McQuery(MC_QUERY_MIN_TIME if kind == "min_time" else MC_QUERY_CHECK, 0,
-                       int(T or 0) & NO_LIMIT)
+        if k >= n:
+            raise IndexError("more queries than models")
+        _QUERY.pack_into(q, k * _QUERY.size, MC_QUERY_MIN_TIME if kind == "min_time" else MC_QUERY_CHECK, 0,
+                         int(T or 0) & NO_LIMIT)
     res = (McBatchResult * n)()
     batch._check(load().mc_batch_run(batch.handle, q, res), "mc_batch_run")
-    return [_batch_result(r) for r in res]
+    return [_batch_result(r) for r in _RESULT.iter_unpack(res)]
 
 
 def mc_batch_trace(batch: Batch, i: int) -> list:
@@ -621,11 +629,18 @@ def mc_batch_get_stats(batch: Batch) -> dict:
     return {k: getattr(st, k) for k, _t in McStats._fields_}
 
 
+# mc_query and mc_batch_result as C lays them out
+_QUERY = struct.Struct("@IIQ")
+_RESULT = struct.Struct("@iIIIQIIQQIIIIQQ")
+assert _QUERY.size == C.sizeof(McQuery) and _RESULT.size == C.sizeof(McBatchResult)
+
+
 def _batch_result(r) -> dict:
-    return {"status": r.status, "kind": "min_time" if r.kind == 1 else "check", "holds": bool(r.holds),
-            "levels": r.levels, "states": r.states, "checks": r.checks, "level": r.level,
-            "time": r.time, "t_ini": r.t_ini, "i": r.wg_index, "j": r.ts_index, "wg": r.wg, "ts": r.ts,
-            "key": r.key[0] | (r.key[1] << 64)}
+    """A result from the fields of an mc_batch_result, in order."""
+    status, kind, holds, levels, states, checks, level, time, t_ini, i, j, wg, ts, lo, hi = r
+    return {"status": status, "kind": "min_time" if kind == 1 else "check", "holds": bool(holds),
+            "levels": levels, "states": states, "checks": checks, "level": level,
+            "time": time, "t_ini": t_ini, "i": i, "j": j, "wg": wg, "ts": ts, "key": lo | (hi << 64)}
 
 
 class Server:
@@ -675,7 +690,7 @@ def mc_server_poll(server: Server, cap: int = 1024, wait_ms: int = 0) -> list:
     out = []
     for k in range(n.value):
         r = buf[k]
-        d = _batch_result(r.result)
+        d = _batch_result(_RESULT.unpack_from(r.result))
         d.update(ticket=r.ticket, submit_s=r.submit_s, admit_s=r.admit_s, done_s=r.done_s,
                  path={0: "loop", 1: "alone", 2: "config"}.get(r.path, "loop"))
         out.append(d)
