@@ -165,6 +165,7 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
   constexpr C kNoneC = (C)~(C)0;
   const uint32_t c_shift = (P - 1 - (unit_ok ? c : 0)) * n_bits;
   const K one_c = (K)1 << c_shift;
+  const K after_c = one_c - 1;  // the count fields of the units after c
   const bool log_on = Q.want_witness != 0;
   const uint64_t seg0 = log_on ? Q.seg[cfg] : 0, seg1 = log_on ? Q.seg[cfg + 1] : 0;
   const uint32_t tmask = tsize - 1;
@@ -195,7 +196,7 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
       S.cnt[(L + 2) % 3] = 0;
       if (early) sc = ld_relaxed_u32(&ctrl->stop_c);
     }
-    if (L > 2)
+    if (greedy && L > 2)
       for (uint32_t x = tid; x < tsize; x += nthr) tcl[x] = (K)0;
     const bool to_terminal = L + 1 == 2 + N;
     for (uint32_t base = 0; base < W; base += spr) {
@@ -218,7 +219,9 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
       if (prune && st > Tc) ok = false;
       const K succ = key + one_c;
       int won = 0;
-      if (ok) {
+      if (!greedy) {
+        won = ok && (key & after_c) == 0;  // no later unit has started: generated here only
+      } else if (ok) {
         const int rc = shared_insert<K>(tnx, tmask, succ);
         if (rc < 0) S.err = (uint32_t)MC_ERR_TABLE_FULL;
         won = rc > 0;
@@ -300,10 +303,9 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
 // (FREE models; the warp units of GREEDY models are wave units, below.)
 // A configuration whose widest level fits one warp (width bound x lanes per
 // state <= 32) is explored by a single warp, its level in registers: state
-// s of the level is held by lanes [s*g, s*g + g), every proposal of the level
-// is in the warp, so duplicates are found exactly by matching the proposed
-// keys across the warp (the lowest lane of equal keys wins), and the winners,
-// ranked by a ballot, become the next level.  No table, no shared counter, no
+// s of the level is held by lanes [s*g, s*g + g), a unit starts only when no
+// later one has started, so a state is proposed once (mc_tree.cu), and the
+// proposals, ranked by a ballot, become the next level.  No table, no shared counter, no
 // block barrier; the same counts, records, log entries and early exit as
 // explore_unit.
 
@@ -369,6 +371,7 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
   const C Tc = T < (uint64_t)(C)~(C)0 ? (C)T : (C)~(C)0;
   const uint32_t c_shift = (P - 1 - (unit_ok ? c : 0)) * n_bits;
   const K one_c = (K)1 << c_shift;
+  const K after_c = one_c - 1;  // the count fields of the units after c
   const bool log_on = Q.want_witness != 0;
   const uint64_t seg0 = log_on ? Q.seg[cfg] : 0, seg1 = log_on ? Q.seg[cfg + 1] : 0;
   const K key2 = ((K)(i + 1) << Q.p.wg_shift) | ((K)(j + 1) << Q.p.ts_shift);
@@ -394,15 +397,8 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
     const C st = nclk > mx ? nclk : mx;  // model time of the successor
     if (prune && st > Tc) ok = false;
     const K succ = key + one_c;
-    // every proposal of the level is in the warp: of equal keys the lowest
-    // lane wins, the others are its duplicates
-    const uint32_t am = __ballot_sync(0xffffffffu, ok);
-    bool won = false;
-    if (ok) {
-      uint32_t peers = __match_any_sync(am, (unsigned long long)KeyOps<K>::lo(succ));
-      if (sizeof(K) == 16) peers &= __match_any_sync(am, (unsigned long long)KeyOps<K>::hi(succ));
-      won = lane == (uint32_t)(__ffs(peers) - 1);
-    }
+    // no later unit has started: the state is generated here only
+    const bool won = ok && (key & after_c) == 0;
     const uint32_t wm = __ballot_sync(0xffffffffu, won);
     const uint32_t Wn = __popc(wm);
     if (won && log_on) {
@@ -743,7 +739,8 @@ __global__ void __launch_bounds__(kCfgMaxThreads) cfg_kernel(const __grid_consta
       S.cut[0] = kNoLevel;
       S.cut[1] = kNoLevel;
     }
-    for (uint32_t x = tid; x < 2 * A.tsize; x += nthr) tab0[x] = (K)0;
+    if (Q.p.rule == MC_GREEDY)  // FREE units keep no table
+      for (uint32_t x = tid; x < 2 * A.tsize; x += nthr) tab0[x] = (K)0;
     __syncthreads();
     const uint64_t T = S.T;
     if (!S.skip) {
