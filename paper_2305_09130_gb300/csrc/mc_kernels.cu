@@ -30,12 +30,13 @@ __global__ void simulate_kernel(const Params p, uint64_t seed, uint32_t walks, u
 // the least (time, walk) over the runs that end at or below the bound goes to
 // *best as (time << 24) | (w - w0).
 template <class C, int PT>
-__global__ void swarm_kernel(const Params p, uint64_t seed, uint64_t w0, uint32_t walks,
+__global__ void swarm_kernel(const Params p, uint64_t seed, uint64_t w0, uint32_t walks, uint32_t per_warp,
                              uint64_t bound, unsigned long long* best) {
-  const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t first = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp;
+  if (first >= walks) return;
+  const uint64_t last = first + per_warp < walks ? first + per_warp : walks;
   const unsigned long long mine =
-      warp_min(swarm_runs<C, PT>(p, seed, w0, gtid, nthreads, walks, bound));
+      warp_min(swarm_runs<C, PT>(p, seed, w0, (uint32_t)first, (uint32_t)last, bound));
   if ((threadIdx.x & 31u) == 0 && mine != kNone) atomicMin(best, mine);
 }
 
@@ -134,10 +135,16 @@ cudaError_t launch_explore(int key_words, int tile, int rule, int scheme, int gr
 
 cudaError_t launch_swarm(const Params& p, uint64_t seed, uint64_t w0, uint32_t walks, uint64_t bound,
                          unsigned long long* best, int grid, cudaStream_t stream) {
+  // a warp takes 256 runs (several rounds of its lanes, so that long and short
+  // runs even out), or as many as the grid's warps need
+  const uint64_t warps = (uint64_t)grid * 8;
+  uint32_t per_warp = 256;
+  if ((uint64_t)per_warp * warps < walks) per_warp = (uint32_t)((walks + warps - 1) / warps);
+  const uint32_t blocks = ((walks + per_warp - 1) / per_warp + 3) / 4;  // 4 warps each
   // the clocks in registers, 32 bits wide where every clock of the model fits
-#define MC_SWARM(PT)                                                                             \
-  (p.clk32 ? swarm_kernel<uint32_t, PT><<<grid, 256, 0, stream>>>(p, seed, w0, walks, bound, best) \
-           : swarm_kernel<uint64_t, PT><<<grid, 256, 0, stream>>>(p, seed, w0, walks, bound, best))
+#define MC_SWARM(PT)                                                                                             \
+  (p.clk32 ? swarm_kernel<uint32_t, PT><<<blocks, 128, 0, stream>>>(p, seed, w0, walks, per_warp, bound, best)   \
+           : swarm_kernel<uint64_t, PT><<<blocks, 128, 0, stream>>>(p, seed, w0, walks, per_warp, bound, best))
   if (p.P <= 4) MC_SWARM(4);
   else if (p.P <= 8) MC_SWARM(8);
   else MC_SWARM(16);
