@@ -69,7 +69,7 @@ WORKLOADS = {
         "(splitmix64 seed 2305091303), speed 1, 128-bit packed states; 1,072,924,481 reachable states "
         "(closed form), widest level 193,344,684",
         "u128", expect=(1, 512, 2), cpu_T=30, ref_T=16,
-        tune={"probe_scheme": ["split", "one_call", "cas_first", "cas_clear"], "stage_chunk": [128, 192],
+        tune={"probe_scheme": ["auto", "split", "one_call", "cas_first", "cas_clear"], "stage_chunk": [128, 192],
               "load_factor_pct": [15, 25]},
         traffic="explore_kernel_c3star_traffic.txt"),
     "c2_star": Workload(
@@ -77,7 +77,7 @@ WORKLOADS = {
         "c2_star: G=80, P=4, WG 2^0..2^8, TS 2^0..2^4, FREE dispatch, cost ceil(WG/TS)*4+WG+2*TS, "
         "speeds U{1..3} (splitmix64 seed 2305091302), 64-bit packed states; 10,385,335 reachable states",
         "u64", expect=(96, 8, 4), cpu_T=None, ref_T=300,
-        tune={"probe_scheme": ["split", "one_call", "cas_first", "cas_clear"], "load_factor_pct": [10, 15],
+        tune={"probe_scheme": ["auto", "split", "one_call", "cas_first", "cas_clear"], "load_factor_pct": [10, 15],
               "stage_chunk": [128, 192]},
         traffic="explore_kernel_c2star_traffic.txt"),
     "c2": Workload(
@@ -93,7 +93,7 @@ WORKLOADS = {
         lambda: W.c3(G=24, rule=W.FREE, key_bits=128),
         "c3 at G=24: P=8, WG 2^0..2^9, TS 2^0..2^5, FREE, cost U{1..16} (seed 2305091303), "
         "128-bit keys (a reduced C3* for profiling: 63,885,179 states)", "u128",
-        tune={"probe_scheme": ["split", "one_call"]}),
+        tune={"probe_scheme": ["auto", "split", "one_call"]}),
 }
 DEFAULT_WORKLOAD = "c3_star"
 METRIC = "unique states/sec"
@@ -101,6 +101,9 @@ UNIT = "states/s"
 FALLBACK_HBM_GBS = 6800.0
 KERNEL_SRCS = [os.path.join(ROOT, "paper_2305_09130_gb300", "csrc", f)
                for f in ("mc_explore.cuh", "mc_device.cuh", "mc_internal.h")]
+# the pass of FREE models whose insert is left to the library ("auto")
+ORDERED_SRCS = KERNEL_SRCS + [os.path.join(ROOT, "paper_2305_09130_gb300", "csrc", f)
+                              for f in ("mc_tree.cu", "mc_tree.h")]
 PROFILES = os.path.join(ROOT, "profiles")
 
 
@@ -207,9 +210,16 @@ def algorithmic_bytes_per_state(P: int, key_words: int) -> int:
     return 32 * P + 32 + 2 * 8 * key_words + 4
 
 
-def kernel_source_hash() -> str:
+def ordered_bytes_per_state(key_words: int) -> int:
+    """Per unique state of the ordered pass, which keeps no visited set: its
+    key written to and read back from the frontier log, and its 4-byte parent
+    index."""
+    return 2 * 8 * key_words + 4
+
+
+def kernel_source_hash(srcs=KERNEL_SRCS) -> str:
     h = hashlib.sha256()
-    for path in KERNEL_SRCS:
+    for path in srcs:
         with open(path, "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -229,14 +239,17 @@ def ncu_traffic_per_launch(path: str, load_factor_pct: int, probe_scheme: str, s
     """DRAM bytes per exploration launch from a committed ncu summary, or
     None when the summary is missing, was taken on another kernel source, or
     holds no capture at this visited-set load factor and probe scheme
-    ("split" or "one_call").  A summary taken on the benchmarked launches
+    ("split", "one_call", ...; "auto", the ordered pass, has sources of its own).  A summary taken on the benchmarked launches
     gives ``dram_bytes_per_launch_lf<LF>_<scheme>``; one taken on a smaller
     case of the same kernel gives ``dram_bytes_per_state_lf<LF>_<scheme>``, scaled
     here by the states one launch processes (the traffic of this DRAM-bound
     kernel grows with the states it inserts)."""
     try:
         fields = read_traffic_file(path)
-        if fields.get("kernel_source_sha256_16") != kernel_source_hash():
+        if probe_scheme == "auto":
+            if fields.get("ordered_source_sha256_16") != kernel_source_hash(ORDERED_SRCS):
+                return None
+        elif fields.get("kernel_source_sha256_16") != kernel_source_hash():
             return None
         key = f"dram_bytes_per_launch_lf{int(load_factor_pct)}_{probe_scheme}"
         if key in fields:
@@ -370,6 +383,12 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
     mc.mc_reserve(model)
     layout = mc.mc_model_layout(model)
     scheme = {v: k for k, v in mc.PROBE.items()}[layout["probe_scheme"]]
+    # FREE models whose insert is left to the library are explored in order,
+    # without a visited set (mc_probe_scheme)
+    ordered = (layout["engine"] == mc.ENGINE["level"] and spec.rule == W.FREE and
+               chosen.get("probe_scheme", 0) == mc.PROBE["auto"])
+    if ordered:
+        scheme = "auto"
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=device)  # > 129 MB of L2
 
     def flush_l2(k):
@@ -425,7 +444,8 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
     value = states_all / (dev_ms_max / 1000.0)
 
     # roofline of the exploration kernel (events on the model's stream)
-    bps = algorithmic_bytes_per_state(spec.P, layout["key_words"])
+    bps = (ordered_bytes_per_state(layout["key_words"]) if ordered
+           else algorithmic_bytes_per_state(spec.P, layout["key_words"]))
     launches = st["explore_launches"]
     states_per_launch = st["states"] / max(launches, 1)
     achieved = bps * st["states"] / (st["explore_ms"] / 1000.0) / 1e9
@@ -438,7 +458,8 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
                 "algorithmic_bytes_per_launch": bps * states_per_launch,
                 "bytes_per_state": bps, "states_per_launch": states_per_launch,
                 "avg_launch_ms": st["explore_ms"] / max(launches, 1),
-                "kernel": (f"explore_kernel<u{64 * layout['key_words']}, tile {1 << (spec.P - 1).bit_length()}, "
+                "kernel": f"tree_kernel<u{64 * layout['key_words']}> (FREE, each state generated once)" if ordered else
+                          (f"explore_kernel<u{64 * layout['key_words']}, tile {1 << (spec.P - 1).bit_length()}, "
                            f"{'FREE' if spec.rule == W.FREE else 'GREEDY'}, {scheme} insert>"
                            if layout["engine"] == mc.ENGINE["level"] else
                            f"cfg_kernel<u{64 * layout['key_words']}> ({layout['unit_threads']} threads per "
@@ -456,7 +477,7 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
     # reads and reads followed by a CAS over a buffer far larger than L2, and
     # reads over one the size of this model's visited set (L2-resident when
     # it fits)
-    if random_roofline:
+    if random_roofline and not ordered:  # (the ordered pass has no random accesses)
         table_bytes = layout["table_slots"] * 8 * layout["key_words"]
         hbm = mc.mc_measure_random_access(64 << 30, 200_000_000, 0)
         hbm_cas = mc.mc_measure_random_access(64 << 30, 200_000_000, 1)
@@ -552,7 +573,7 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
                    "options_fixed": fixed,
                    "probe_scheme": scheme,
                    "load_factor_pct": layout_lf(opts),
-                   "visited_set_bytes": layout["table_slots"] * 8 * layout["key_words"],
+                   "visited_set_bytes": 0 if ordered else layout["table_slots"] * 8 * layout["key_words"],
                    "frontier_log_bytes": layout["log_capacity"] * (8 * layout["key_words"] + 4),
                    "states_per_step": states_local / steps,
                    "checks_per_step": r["checks"]},
@@ -737,7 +758,7 @@ def run_pe(args):
     fd, cache = tempfile.mkstemp(suffix=".json")
     os.close(fd)
     tuned = AT.tune_pe(spec, "count" if args.query == "count" else "min_time",
-                       space={"lanes_per_state": [8, 16, 32], "blocks_per_sm": [0, 2, 3]}, reps=1, path=cache)
+                       space={"blocks_per_sm": [0, 1]}, reps=1, path=cache)
     os.unlink(cache)
     opts = mc.mc_options_default(timing=1, **tuned["options"])
     stream = torch.cuda.Stream(device)
@@ -783,11 +804,10 @@ def run_pe(args):
     dev_ms_max = reduce_scalar(dev_ms, "max", device)
     states_all = reduce_scalar(st["states"], "sum", device)
     value = states_all / (dev_ms_max / 1000.0)
-    # per unique state: one 32-byte bucket probe per generated successor, one
-    # 32-byte slot write-back, the 16-byte key written to and read back from
-    # the frontier log, the 4-byte parent index
+    # per unique state (each generated once, no visited set): the 16-byte key
+    # written to and read back from the frontier log, the 4-byte parent index
     probes_per_state = st["probes"] / max(st["states"], 1)
-    bps = 32 * probes_per_state + 32 + 2 * 16 + 4
+    bps = 2 * 16 + 4
     launches = st["explore_launches"]
     achieved = bps * st["states"] / (st["explore_ms"] / 1000.0) / 1e9
     peak, peak_kind = measured_hbm_peak()
@@ -796,12 +816,11 @@ def run_pe(args):
                 "algorithmic_bytes_per_launch": bps * st["states"] / max(launches, 1),
                 "avg_launch_ms": st["explore_ms"] / max(launches, 1),
                 "levels_per_launch": st["device_steps"] / max(launches, 1),
-                "kernel": f"pe_explore_kernel<tile {lay['tile']}>",
+                "kernel": "pe_ordered_kernel",
                 "peak_source": f"{peak_kind} HBM copy bandwidth"}
     # end to end through the public C-ABI from host buffers
     e2e_s, h2d, d2h = [], 0, 0
-    big = dict(tuned["options"], log_capacity=lay["log_capacity"],
-               table_log2=lay["table_slots"].bit_length() - 1)
+    big = dict(tuned["options"], log_capacity=lay["log_capacity"])
     for k in range(args.steps):
         torch.cuda.synchronize()
         t0 = time.perf_counter()

@@ -54,6 +54,8 @@ CONFIG_SPACE = {
     "unit_threads": [0, 128, 256, 512],
     "lanes_per_state": [0, 16],
 }
+# FREE models on the level engine in order: no insert, no visited set
+ORDERED_SPACE = {"engine": [1], "probe_scheme": [0], "blocks_per_sm": [0]}
 BATCH_LEVEL_SPACE = {"engine": [1], "blocks_per_sm": [0, 1, 2], "load_factor_pct": [25, 50]}
 BATCH_CONFIG_SPACE = {"engine": [2], "unit_threads": [0, 256, 512], "lanes_per_state": [0, 8]}
 
@@ -150,6 +152,8 @@ def tune_query(spec, query: str = "min_time", T: Optional[int] = None, space=Non
     cache = load_cache(path) if cache is None else cache
     if space is None:  # both engines where the configuration engine takes the model
         space = [LEVEL_SPACE] + ([CONFIG_SPACE] if lay["engine"] == mc.ENGINE["config"] else [])
+        if spec.rule == mc.MC_FREE:
+            space.append(ORDERED_SPACE)
 
     def measure(c):
         m = mc.mc_model_create(spec, mc.mc_options_default(timing=1, **c))
@@ -234,7 +238,7 @@ def tune_pe(spec, query: str = "min_time", space=None, reps: int = 2, cache: Opt
         run()
         if not grown:  # later candidates start at the grown buffer sizes
             L = mc.mc_pe_model_layout(m)
-            grown.update(log_capacity=L["log_capacity"], table_log2=L["table_slots"].bit_length() - 1)
+            grown.update(log_capacity=L["log_capacity"])
         mc.mc_pe_reset_stats(m)
         ans = run()
         ms = mc.mc_pe_get_stats(m)["explore_ms"]
