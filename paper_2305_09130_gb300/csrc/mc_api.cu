@@ -237,6 +237,8 @@ struct mc_model {
   size_t cfg_smem = 0;
   bool cfg_warp = false;  // one warp per configuration: wave units (GREEDY), or the widest level's lanes fit a warp
   int cfg_unit_threads = 0;  // mc_layout.unit_threads
+  uint32_t cfg_segment = 0;  // wave units: work-groups of a segment (0: no wave units)
+  uint64_t cfg_units = 0;    // units of a pass: configurations, or their segments
   // device state
   bool reserved = false;
   int device = -1;
@@ -538,11 +540,20 @@ int size_buffers(mc_model* m) {
     // subsets fit it (wave units), whatever its lanes per state
     m->cfg_warp = fits_warp || mc::wave_model(m->rule, m->P, m->opt.unit_threads);
     m->cfg_threads = m->cfg_warp ? (int)mc::kCfgWarpBlockThreads : m->cfg_unit_threads;
+    m->cfg_segment = 0;
+    m->cfg_units = ab;
+    if (mc::wave_model(m->rule, m->P, m->opt.unit_threads)) {
+      m->cfg_segment = mc::wave_segment(m->max_level - 2);
+      if (m->cfg_segment) {
+        m->cfg_units = 0;
+        for (uint32_t n : m->N) m->cfg_units += mc::wave_segments(n, m->cfg_segment);
+      }
+    }
     const uint64_t key_bytes = 8ull * m->key_words;
     const uint64_t ctrl_bytes = (mc::kBarBytes + sizeof(Ctrl)) * kSlots + kScalarBytes + 8ull * (m->max_level + 2) * 5;
     uint64_t total = mul_sat(m->log_cap, key_bytes + 4);
     total = add_sat(total, ctrl_bytes + 4ull * (2 * ab + m->P));
-    total = add_sat(total, 8 * (ab + 1) + 2 * sizeof(mc::CfgRec) * ab + 4 * ab + 24 * ab + 8 * sizeof(mc::CfgPass));
+    total = add_sat(total, 8 * (ab + 2) + 2 * sizeof(mc::CfgRec) * ab + 28 * m->cfg_units + 8 * sizeof(mc::CfgPass));
     total = add_sat(total, 16ull * (m->max_level + 2) * kSlots);  // level widths per result slot
     m->device_bytes = total;
     return MC_OK;
@@ -652,7 +663,7 @@ int reserve(mc_model* m) {
     if (m->opt.blocks_per_sm) bps = std::min<int>(bps, (int)m->opt.blocks_per_sm);
     m->cfg_grid_max = sms * bps;
     const uint64_t per_block = m->cfg_warp ? (uint64_t)m->cfg_threads / 32 : 1;
-    m->cfg_grid = (int)std::min<uint64_t>((ab + per_block - 1) / per_block, (uint64_t)sms * bps);
+    m->cfg_grid = (int)std::min<uint64_t>((m->cfg_units + per_block - 1) / per_block, (uint64_t)sms * bps);
   }
 
   const uint64_t key_bytes = 8ull * m->key_words;
@@ -667,12 +678,12 @@ int reserve(mc_model* m) {
   const size_t ctrl_bytes = mc::kBarBytes * kSlots + mirror_bytes + 16 * L2 + 8 * L2;
   m->d_ctrl_block = (uint8_t*)dev_alloc(m, ctrl_bytes);
   if (cfg) {
-    m->d_seg = (uint64_t*)dev_alloc(m, 8 * (ab + 1));
+    m->d_seg = (uint64_t*)dev_alloc(m, 8 * (ab + 2));
     m->d_rec = (mc::CfgRec*)dev_alloc(m, 2 * sizeof(mc::CfgRec) * ab);  // two passes at once
-    m->d_order = (uint32_t*)dev_alloc(m, 4 * ab);
+    m->d_order = (uint32_t*)dev_alloc(m, 4 * m->cfg_units);
     m->d_cfg_levels = (uint64_t*)dev_alloc(m, 16 * L2 * kSlots);
     m->d_pair_pass = (mc::CfgPass*)dev_alloc(m, 8 * sizeof(mc::CfgPass));
-    m->d_pair_units = (uint64_t*)dev_alloc(m, 8 * 3 * ab);
+    m->d_pair_units = (uint64_t*)dev_alloc(m, 8 * 3 * m->cfg_units);
   }
   if (!m->d_params || (table && !m->d_table) || !m->d_log_keys || !m->d_log_par || !m->d_ctrl_block ||
       (cfg && (!m->d_seg || !m->d_rec || !m->d_order || !m->d_cfg_levels || !m->d_pair_pass ||
@@ -704,10 +715,11 @@ int reserve(mc_model* m) {
   // configuration engine, the segment starts and the order)
   const size_t o_params = align_up(mirror_bytes, 64);
   const size_t o_seg = align_up(o_params + np * 4, 8);
-  const size_t o_order = o_seg + (cfg ? 8 * (ab + 1) : 0);
-  const size_t o_pair = align_up(o_order + (cfg ? 4 * ab : 0), 64);
+  const uint64_t units = m->cfg_units;
+  const size_t o_order = o_seg + (cfg ? 8 * (ab + 2) : 0);
+  const size_t o_pair = align_up(o_order + (cfg ? 4 * units : 0), 64);
   const size_t o_pair_units = o_pair + (cfg ? 8 * sizeof(mc::CfgPass) : 0);
-  m->h_block_bytes = o_pair_units + (cfg ? 8 * 3 * ab : 0);
+  m->h_block_bytes = o_pair_units + (cfg ? 8 * 3 * units : 0);
   m->h_block = (uint8_t*)mc::pinned_alloc(m->h_block_bytes);
   if (!m->h_block) {
     release(m);
@@ -732,10 +744,16 @@ int reserve(mc_model* m) {
     uint64_t* h_seg = (uint64_t*)(m->h_block + o_seg);
     uint32_t* h_order = (uint32_t*)(m->h_block + o_order);
     std::copy(m->seg.begin(), m->seg.end(), h_seg);
-    std::copy(m->order.begin(), m->order.end(), h_order);
-    MC_CUDA(m, cudaMemcpyAsync(m->d_seg, h_seg, 8 * (ab + 1), cudaMemcpyHostToDevice, m->stream));
-    MC_CUDA(m, cudaMemcpyAsync(m->d_order, h_order, 4 * ab, cudaMemcpyHostToDevice, m->stream));
-    m->stats.h2d_bytes += 12 * ab + 8;
+    h_seg[ab + 1] = units;
+    // the units of a pass: configurations, or (part << 24 | configuration)
+    uint64_t x = 0;
+    for (uint32_t c : m->order) {
+      const uint64_t parts = m->cfg_segment ? mc::wave_segments(m->N[c], m->cfg_segment) : 1;
+      for (uint64_t part = 0; part < parts; ++part) h_order[x++] = (uint32_t)(part << 24) | c;
+    }
+    MC_CUDA(m, cudaMemcpyAsync(m->d_seg, h_seg, 8 * (ab + 2), cudaMemcpyHostToDevice, m->stream));
+    MC_CUDA(m, cudaMemcpyAsync(m->d_order, h_order, 4 * units, cudaMemcpyHostToDevice, m->stream));
+    m->stats.h2d_bytes += 8 * (ab + 2) + 4 * units;
   }
 
   Params& p = m->params;
@@ -756,7 +774,7 @@ int reserve(mc_model* m) {
       const int c = k & 1;  // 0: certificate at T_min - 1, 1: counterexample at T_min
       Q.T_src = m->d_tmin;
       Q.T_delta = c == 0 ? -1 : 0;
-      Q.group = m->tile;
+      Q.group = (uint32_t)m->tile | m->cfg_segment << 8;
       Q.log_keys = m->d_log_keys;
       Q.log_par = m->d_log_par;
       Q.seg = m->d_seg;
@@ -767,14 +785,15 @@ int reserve(mc_model* m) {
       Q.want_witness = c == 1;
     }
     uint64_t* hu = (uint64_t*)(m->h_block + o_pair_units);
-    for (uint64_t x = 0; x < ab; ++x) {
-      hu[2 * x] = m->order[x];                        // certificate
-      hu[2 * x + 1] = (1ull << 32) | m->order[x];     // counterexample
-      hu[2 * ab + x] = (1ull << 32) | m->order[x];    // counterexample alone
+    const uint32_t* h_order = (const uint32_t*)(m->h_block + o_order);
+    for (uint64_t x = 0; x < units; ++x) {
+      hu[2 * x] = h_order[x];                          // certificate
+      hu[2 * x + 1] = (1ull << 32) | h_order[x];       // counterexample
+      hu[2 * units + x] = (1ull << 32) | h_order[x];   // counterexample alone
     }
     MC_CUDA(m, cudaMemcpyAsync(m->d_pair_pass, hp, 8 * sizeof(mc::CfgPass), cudaMemcpyHostToDevice, m->stream));
-    MC_CUDA(m, cudaMemcpyAsync(m->d_pair_units, hu, 8 * 3 * ab, cudaMemcpyHostToDevice, m->stream));
-    m->stats.h2d_bytes += 8 * sizeof(mc::CfgPass) + 24 * ab;
+    MC_CUDA(m, cudaMemcpyAsync(m->d_pair_units, hu, 8 * 3 * units, cudaMemcpyHostToDevice, m->stream));
+    m->stats.h2d_bytes += 8 * sizeof(mc::CfgPass) + 24 * units;
   }
   m->reserved = true;
   return MC_OK;
@@ -824,7 +843,7 @@ int enqueue_cfg_pass(mc_model* m, uint64_t T, const uint64_t* T_src, int64_t del
   Q.prune = prune;
   Q.early_exit = early_exit;
   Q.want_witness = witness;
-  Q.group = m->tile;
+  Q.group = (uint32_t)m->tile | m->cfg_segment << 8;
   Q.log_keys = m->d_log_keys;
   Q.log_par = m->d_log_par;
   Q.seg = m->d_seg;
@@ -837,7 +856,7 @@ int enqueue_cfg_pass(mc_model* m, uint64_t T, const uint64_t* T_src, int64_t del
   L.wcap = m->cfg_wcap;
   L.tsize = m->cfg_tsize;
   if (m->cfg_warp) {  // every block serves warp units
-    L.n_wunits = (uint64_t)m->a * m->b;
+    L.n_wunits = m->cfg_units;
     L.wnext = &Q.ctrl->units_next;
     L.warp_blocks = (uint32_t)m->cfg_grid;
   } else {
@@ -858,7 +877,7 @@ int enqueue_cfg_pass(mc_model* m, uint64_t T, const uint64_t* T_src, int64_t del
 // 1, unless refine is off) and the counterexample check at T_min (slot 2)
 // in one launch; T_min is read on the device from the min pass.
 int enqueue_cfg_pair(mc_model* m, bool prune, bool early_exit, bool refine) {
-  const uint64_t ab = (uint64_t)m->a * m->b;
+  const uint64_t ab = m->cfg_units;
   MC_CUDA(m, cudaMemsetAsync(cfg_levels_at(m, 1), 0, 2 * 16ull * (m->max_level + 2), m->stream));
   mc::CfgLaunch L{};
   L.passes = m->d_pair_pass + 2 * ((prune ? 2 : 0) + (early_exit ? 1 : 0));  // descriptors per option pair

@@ -593,6 +593,7 @@ __device__ void cfg_epilogue_warp(const CfgPass& Q, uint64_t T) {
       best = v < best ? v : best;
     }
   }
+  if (wave_unit(p)) deep = max(deep, ld_relaxed_u32(&Q.ctrl->pad1[0]));  // (wave units' records leave it out)
   deep = __reduce_max_sync(0xffffffffu, deep);
   stop = __reduce_min_sync(0xffffffffu, stop);
   best = warp_min_u64(best);
@@ -636,7 +637,11 @@ __device__ void warp_role(const CfgLaunch& A) {
     if (u >= n) return;
     const uint64_t code = A.wunits ? __ldg(A.wunits_rev ? A.wunits - u : A.wunits + u) : 0ull;
     const CfgPass& Q = A.wunits ? A.passes[code >> 32] : A.one;
-    const uint32_t cfg = A.wunits ? (uint32_t)code : __ldg(Q.order + u);
+    // a configuration, or (wave units of a single model: Q.group holds the
+    // segments' length above the lanes per state) a segment of one
+    const uint32_t part = A.wunits ? (uint32_t)code : __ldg(Q.order + u);
+    const uint32_t segment = Q.group >> 8;
+    const uint32_t cfg = segment ? part & 0xFFFFFFu : part;
     // the threshold, as for a block unit
     unsigned long long t = 0;
     uint32_t skip = 0;
@@ -652,8 +657,8 @@ __device__ void warp_role(const CfgLaunch& A) {
     t = __shfl_sync(0xffffffffu, t, 0);
     skip = __shfl_sync(0xffffffffu, skip, 0);
     if (!skip && wave_unit(Q.p)) {
-      if (Q.p.clk32) explore_wave<K, uint32_t>(Q, cfg, t);
-      else explore_wave<K, uint64_t>(Q, cfg, t);
+      if (Q.p.clk32) explore_wave<K, uint32_t>(Q, cfg, t, segment, segment ? part >> 24 : 0u);
+      else explore_wave<K, uint64_t>(Q, cfg, t, segment, segment ? part >> 24 : 0u);
     } else if (!skip) {
       const uint32_t err = Q.p.clk32 ? explore_unit_warp<K, uint32_t>(Q, cfg, t)
                                      : explore_unit_warp<K, uint64_t>(Q, cfg, t);
@@ -665,7 +670,8 @@ __device__ void warp_role(const CfgLaunch& A) {
     if (lane == 0) {
       __threadfence();
       const uint32_t done = atomicAdd(&Q.ctrl->units_done, 1u) + 1;
-      last = done == Q.p.a * Q.p.b;
+      const uint32_t ab = Q.p.a * Q.p.b;
+      last = done == (segment ? (uint32_t)__ldg(Q.seg + ab + 1) : ab);  // (segments: their number follows the starts)
       if (last) __threadfence();
     }
     last = __shfl_sync(0xffffffffu, last, 0);

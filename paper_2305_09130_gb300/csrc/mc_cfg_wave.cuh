@@ -19,6 +19,12 @@
 // the bound already): a unit whose next clock passes T starts in no state, so
 // the wave ends early and the search with it.
 //
+// The chain can be entered at any wave: before instant m unit c has started
+// ceil(m / t_c) times (each of its starts is a multiple of t_c), and that state
+// was reached if none of those starts ended beyond T.  So a configuration's
+// levels can be split into segments explored at the same time; the wave on a
+// border is explored on both sides, and each side counts its own levels.
+//
 // Positions in the bitmap: the units of E in descending index, so the order
 // of the bitmap's indices is the order of the packed keys and the smallest
 // key is the lowest bit.  Bits 0-4 of an index pick the bit of a lane's word,
@@ -30,9 +36,11 @@
 // barrier to every level.  Measured on GB300, counting C3 literal (10 x 6
 // configurations of up to 4,096 work-groups, 8 units of one speed, 128-bit
 // keys): the pass 4,550 us with block units (a hashed table in shared memory
-// and a block barrier per level), 324 us here; C2 literal's pass (4 units of
-// uneven speeds, 1,024 work-groups, almost every wave one unit) 422 -> 94 us.
-// Left: 31 instructions per level at 5 cycles each, one warp to a scheduler.
+// and a block barrier per level), 324 us with a warp per configuration, about
+// 50 us with a warp per segment; C2 literal's pass (4 units of uneven speeds,
+// 1,024 work-groups, almost every wave one unit) 422, 94 and 33 us.  Left: a
+// launch's fixed costs, and 31 instructions per level at 5 cycles each, one
+// warp to a scheduler.
 #pragma once
 #include <cstdint>
 
@@ -104,7 +112,9 @@ __device__ __forceinline__ uint32_t wave_full(uint32_t lane) {
 // may start (pruning, or the work-groups run out): returns the last level's
 // subsets.  The levels are not empty: a subset smaller than A leaves a unit
 // to start.  Rare (a configuration's last wave), so not specialised.
-__device__ __forceinline__ uint32_t wave_part(uint32_t A, uint32_t m, uint32_t lane, unsigned long long* level) {
+// Levels from .. to - 1 of them are counted.
+__device__ __forceinline__ uint32_t wave_part(uint32_t A, uint32_t m, uint32_t lane, unsigned long long* level,
+                                              uint32_t from, uint32_t to) {
   uint32_t keep[5], up[5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
@@ -116,7 +126,7 @@ __device__ __forceinline__ uint32_t wave_part(uint32_t A, uint32_t m, uint32_t l
   for (uint32_t x = 0; x < m; ++x) {
     cur = A >> 5 ? wave_step<5>(cur, keep, up) : wave_step<0>(cur, keep, up);
     const uint32_t w = __reduce_add_sync(0xffffffffu, __popc(cur));
-    if (lane == 0) atomicAdd(level + 2 * x, (unsigned long long)w);
+    if (lane == 0 && x >= from && x < to) atomicAdd(level + 2 * x, (unsigned long long)w);
   }
   return cur;
 }
@@ -143,6 +153,29 @@ struct WaveClocks {
       t[c] = unit ? (C)((uint64_t)__ldg(p.cost + cfg) * __ldg(p.speed + c)) : (C)0;
       clk[c] = unit ? (C)0 : (C)~(C)0;  // never the smallest
     }
+  }
+  // The state before the wave in which the work-group after the first `k`
+  // starts (its instant by bisection: the smallest with more than k starts at
+  // or before it); returns the work-groups taken by then.
+  __device__ uint32_t enter(const Params& p, uint32_t k) {
+    C t_min = t[0];
+    for (int c = 1; c < PT; ++c) t_min = c < (int)p.P && t[c] < t_min ? t[c] : t_min;
+    C lo = 0, hi = (C)k * t_min;
+    while (lo < hi) {
+      const C mid = lo + (hi - lo) / 2;
+      uint64_t starts = 0;
+      for (int c = 0; c < PT; ++c) starts += c < (int)p.P ? (uint64_t)(mid / t[c]) + 1 : 0ull;
+      if (starts > k) hi = mid;
+      else lo = mid + 1;
+    }
+    uint32_t before = 0;
+    for (int c = 0; c < PT; ++c) {
+      if (c >= (int)p.P) continue;
+      const C n = lo / t[c] + (lo % t[c] ? 1 : 0);
+      clk[c] = n * t[c];
+      before += (uint32_t)n;
+    }
+    return before;
   }
   // E: the units whose clock is the smallest; late: those of them whose next
   // clock passes `bound`
@@ -202,6 +235,22 @@ struct WaveClocks<C, 0> {
     clk = unit ? (C)0 : (C)~(C)0;
     nxt = clk + t;
   }
+  __device__ uint32_t enter(const Params&, uint32_t k) {
+    const C t_min = lanes_min(unit ? t : (C)~(C)0);
+    C lo = 0, hi = (C)k * t_min;
+    while (lo < hi) {
+      const C mid = lo + (hi - lo) / 2;
+      // (a unit's starts are capped, so that 32 bits hold the sum)
+      const C q = mid / t;
+      const uint32_t starts = __reduce_add_sync(0xffffffffu, !unit ? 0u : (uint32_t)(q < (C)k ? q : (C)k) + 1);
+      if (starts > k) hi = mid;
+      else lo = mid + 1;
+    }
+    const C n = unit ? lo / t + (lo % t ? 1 : 0) : (C)0;
+    if (unit) clk = n * t;
+    nxt = clk + t;
+    return __reduce_add_sync(0xffffffffu, (uint32_t)n);
+  }
   __device__ __forceinline__ void first(C bound, uint32_t& E, uint32_t& late) {
     const C mn = lanes_min(clk);  // (every lane takes part)
     in = unit && clk == mn;
@@ -227,10 +276,11 @@ __device__ __forceinline__ uint32_t wave_positions(uint32_t E, uint32_t mask) {
   return A;
 }
 
-// Explore configuration `cfg` of pass Q at threshold T with one warp: the
-// same widths, record and early exit as explore_unit.
+// Explore work-groups k0 + 1 .. k1 of configuration `cfg` of pass Q at
+// threshold T with one warp (the whole configuration: 0 .. N): the same
+// widths, record and early exit as explore_unit.
 template <class K, class C, int PT>
-__device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T) {
+__device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, uint32_t k0, uint32_t k1) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t P = Q.p.P, b = Q.p.b;
   const uint32_t i = cfg / b, j = cfg % b;
@@ -243,22 +293,27 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T) {
   unsigned long long* const levels = reinterpret_cast<unsigned long long*>(Q.levels);
   Ctrl* const ctrl = Q.ctrl;
 
-  uint32_t sum = 0;              // work-groups taken before the current wave
+  // work-groups taken before the current wave; the first wave's may have
+  // started before the segment
+  uint32_t sum = k0 ? clocks.enter(Q.p, k0) : 0u;
+  const bool reached = k0 == 0 || clocks.largest(P) <= Tc;
   uint32_t E = 0, cur = 0;       // the wave's units, the current level's subsets
-  uint32_t ones = 0, window = 0; // one-state levels of the current 32-level window
+  uint32_t ones = 0;             // one-state levels of the current 32-level window
+  uint32_t window = (3 + sum) >> 5;
   bool done = false;             // the terminal level was reached
   // early exit: the least level known to hold a violating terminal, asked
   // for at the end of a window and used at the next, so the load never holds
   // a level up (a later stop only explores levels that are not counted)
   uint32_t asked = early ? ld_relaxed_u32(&ctrl->stop_c) : 0u;
-  for (;;) {
+  const bool beyond = k0 && asked && ~asked <= 2 + k0;  // below the first violating level: not counted
+  while (reached && !beyond && sum < k1) {
     uint32_t late = 0;
     // waves of one unit, the common ones of uneven speeds: one state per
     // level, one branch per wave; their widths are added window by window
     for (;;) {
       clocks.first(Tc, E, late);
       const uint32_t at = 3 + sum;  // the wave's first level
-      if ((E & (E - 1)) | late | (uint32_t)(sum + 1 == N) | (uint32_t)((at >> 5) != window)) break;
+      if ((E & (E - 1)) | late | (uint32_t)(sum + 1 >= k1) | (uint32_t)((at >> 5) != window)) break;
       ones |= 1u << (at & 31u);
       ++sum;
       clocks.advance();
@@ -289,13 +344,15 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T) {
         case 9: width = wave_full<9>(lane); break;
         default: width = wave_full<10>(lane); break;
       }
-      if (lane < e) atomicAdd(levels + 2ull * (before + 1 + lane), (unsigned long long)width);
+      // (a wave on the segment's border: its own levels only)
+      if (lane < e && sum + lane >= k0 && sum + lane < k1)
+        atomicAdd(levels + 2ull * (before + 1 + lane), (unsigned long long)width);
       sum += e;
       clocks.advance();
     } else {  // the last wave: the work-groups run out, or pruning keeps a unit from starting
       const uint32_t A = wave_positions(E, E & ~late);
       const uint32_t m = min(N - sum, (uint32_t)__popc(A));
-      cur = wave_part(A, m, lane, levels + 2ull * (before + 1));
+      cur = wave_part(A, m, lane, levels + 2ull * (before + 1), k0 > sum ? k0 - sum : 0u, k1 - sum);
       sum += m;
       done = sum == N;
       break;
@@ -333,22 +390,28 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T) {
       }
     }
   }
-  if (lane == 0) {
+  // (pad1[0]: the deepest level any unit of the pass reached)
+  if (lane == 0 && reached) atomicMax(&ctrl->pad1[0], 2 + min(sum, k1));
+  if (lane == 0 && k1 == N) {
     if (hit && early) atomicMax(&ctrl->stop_c, ~(2u + N));
     CfgRec rec;
     rec.vpack = hit ? pack_tij((uint64_t)tv, i, j) : kNone;
     rec.wkey_lo = hit ? KeyOps<K>::lo(key) : kNone;
     rec.wkey_hi = hit ? KeyOps<K>::hi(key) : kNone;
     rec.widx = 0;  // no log: wave_trace gives the path
-    rec.deepest = 2 + sum;
+    rec.deepest = 0;
     Q.rec[cfg] = rec;
   }
 }
 
+// Segment number `part` of a configuration (`segment` work-groups each, 0: the
+// whole configuration).
 template <class K, class C>
-__device__ __forceinline__ void explore_wave(const CfgPass& Q, uint32_t cfg, uint64_t T) {
-  if (Q.p.P <= 2) explore_unit_wave<K, C, 2>(Q, cfg, T);
-  else explore_unit_wave<K, C, 0>(Q, cfg, T);
+__device__ __forceinline__ void explore_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, uint32_t segment, uint32_t part) {
+  const uint32_t N = __ldg(Q.p.N + cfg), k0 = segment * part;
+  const uint32_t k1 = segment && N - k0 > segment ? k0 + segment : N;
+  if (Q.p.P <= 2) explore_unit_wave<K, C, 2>(Q, cfg, T, k0, k1);
+  else explore_unit_wave<K, C, 0>(Q, cfg, T, k0, k1);
 }
 
 // The trace s0 -> the witness of configuration (i, j), replayed by one warp:

@@ -23,4 +23,20 @@ inline bool wave_model(uint32_t rule, uint32_t P, uint32_t unit_threads) {
   return rule == MC_GREEDY && P <= kWaveMaxP && unit_threads == 0;
 }
 
+// A single model's launch splits a configuration's levels into segments of
+// this many work-groups (more when a configuration would have over 255), each
+// explored by a warp of its own: the state in which every wave before an
+// instant has run is known (see mc_cfg_wave.cuh), so segments need not wait
+// for each other.  C3 literal's configurations of 4,096 work-groups are 32
+// warps instead of one.  (Runs of many models have warps enough and take a
+// configuration whole.)
+constexpr uint32_t kWaveSegment = 128;
+
+inline uint32_t wave_segment(uint32_t n_max) {
+  if (n_max >= 1u << 27) return 0;  // (the search for a segment's start sums starts in 32 bits)
+  const uint32_t least = (uint32_t)(((uint64_t)n_max + 254) / 255);
+  return least > kWaveSegment ? least : kWaveSegment;
+}
+inline uint64_t wave_segments(uint32_t n, uint32_t segment) { return ((uint64_t)n + segment - 1) / segment; }
+
 }  // namespace mc

@@ -91,7 +91,8 @@ def gpu_models():
         out.append(W.random_small(7330 + P, P, 2, 2, 19 if P < 9 else 12, cost_max=7, speed_max=3, rule=W.GREEDY))
     # hundreds of levels, waves of one unit and of several mixed (the widths of
     # one-state levels are added 32 levels at a time)
-    for P, speed in ((2, [2, 3]), (3, [2, 3, 3]), (5, [1, 2, 2, 3, 3])):
+    # (and several segments of a configuration, their borders inside waves)
+    for P, speed in ((2, [2, 3]), (3, [2, 3, 3]), (5, [1, 2, 2, 3, 3]), (6, [2] * 6)):
         deep = W.random_small(7390 + P, P, 2, 2, 300, cost_max=5, rule=W.GREEDY)
         deep.speed = speed
         deep.n_workgroups = [300, 257, 33, 100]
