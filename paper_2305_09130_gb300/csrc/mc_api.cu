@@ -553,7 +553,7 @@ int size_buffers(mc_model* m) {
     const uint64_t ctrl_bytes = (mc::kBarBytes + sizeof(Ctrl)) * kSlots + kScalarBytes + 8ull * (m->max_level + 2) * 5;
     uint64_t total = mul_sat(m->log_cap, key_bytes + 4);
     total = add_sat(total, ctrl_bytes + 4ull * (2 * ab + m->P));
-    total = add_sat(total, 8 * (ab + 2) + 2 * sizeof(mc::CfgRec) * ab + 28 * m->cfg_units + 8 * sizeof(mc::CfgPass));
+    total = add_sat(total, 8 * (ab + 1) + 2 * sizeof(mc::CfgRec) * ab + 28 * m->cfg_units + 8 * sizeof(mc::CfgPass));
     total = add_sat(total, 16ull * (m->max_level + 2) * kSlots);  // level widths per result slot
     m->device_bytes = total;
     return MC_OK;
@@ -678,7 +678,7 @@ int reserve(mc_model* m) {
   const size_t ctrl_bytes = mc::kBarBytes * kSlots + mirror_bytes + 16 * L2 + 8 * L2;
   m->d_ctrl_block = (uint8_t*)dev_alloc(m, ctrl_bytes);
   if (cfg) {
-    m->d_seg = (uint64_t*)dev_alloc(m, 8 * (ab + 2));
+    m->d_seg = (uint64_t*)dev_alloc(m, 8 * (ab + 1));
     m->d_rec = (mc::CfgRec*)dev_alloc(m, 2 * sizeof(mc::CfgRec) * ab);  // two passes at once
     m->d_order = (uint32_t*)dev_alloc(m, 4 * m->cfg_units);
     m->d_cfg_levels = (uint64_t*)dev_alloc(m, 16 * L2 * kSlots);
@@ -716,7 +716,7 @@ int reserve(mc_model* m) {
   const size_t o_params = align_up(mirror_bytes, 64);
   const size_t o_seg = align_up(o_params + np * 4, 8);
   const uint64_t units = m->cfg_units;
-  const size_t o_order = o_seg + (cfg ? 8 * (ab + 2) : 0);
+  const size_t o_order = o_seg + (cfg ? 8 * (ab + 1) : 0);
   const size_t o_pair = align_up(o_order + (cfg ? 4 * units : 0), 64);
   const size_t o_pair_units = o_pair + (cfg ? 8 * sizeof(mc::CfgPass) : 0);
   m->h_block_bytes = o_pair_units + (cfg ? 8 * 3 * units : 0);
@@ -744,16 +744,16 @@ int reserve(mc_model* m) {
     uint64_t* h_seg = (uint64_t*)(m->h_block + o_seg);
     uint32_t* h_order = (uint32_t*)(m->h_block + o_order);
     std::copy(m->seg.begin(), m->seg.end(), h_seg);
-    h_seg[ab + 1] = units;
+    if (m->cfg_segment) h_seg[0] = units;  // (wave units keep no log)
     // the units of a pass: configurations, or (part << 24 | configuration)
     uint64_t x = 0;
     for (uint32_t c : m->order) {
       const uint64_t parts = m->cfg_segment ? mc::wave_segments(m->N[c], m->cfg_segment) : 1;
       for (uint64_t part = 0; part < parts; ++part) h_order[x++] = (uint32_t)(part << 24) | c;
     }
-    MC_CUDA(m, cudaMemcpyAsync(m->d_seg, h_seg, 8 * (ab + 2), cudaMemcpyHostToDevice, m->stream));
+    MC_CUDA(m, cudaMemcpyAsync(m->d_seg, h_seg, 8 * (ab + 1), cudaMemcpyHostToDevice, m->stream));
     MC_CUDA(m, cudaMemcpyAsync(m->d_order, h_order, 4 * units, cudaMemcpyHostToDevice, m->stream));
-    m->stats.h2d_bytes += 8 * (ab + 2) + 4 * units;
+    m->stats.h2d_bytes += 8 * (ab + 1) + 4 * units;
   }
 
   Params& p = m->params;

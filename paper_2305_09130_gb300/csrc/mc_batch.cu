@@ -861,7 +861,7 @@ int breserve_cfg(mc_batch* b) {
   b->cfg_wcap = 32;
   bool block_models = false;
   for (const mc::CfgModelPrep& M : b->cm) {
-    units += M.ab;
+    units += M.units;
     if (mc::cfg_warp_model(M, b->opt)) continue;  // a warp per configuration: no block shape
     block_models = true;
     b->cfg_threads = std::max<int>(b->cfg_threads, (int)M.threads);
@@ -1052,7 +1052,7 @@ int mc_batch_create(const mc_model_desc* descs, uint32_t n, const mc_options* op
       }
       b->pool_off[i] = off;
       off += b->cm[i].region;
-      units += b->cm[i].ab;
+      units += b->cm[i].units;
       b->wg[i] = b->cm[i].wg;
       b->ts[i] = b->cm[i].ts;
     }
@@ -1927,12 +1927,11 @@ int mc_server_submit(mc_server* S, const mc_model_desc* desc, const mc_query* q,
   int rc = MC_ERR_INVAL;
   if (S->opt.engine != MC_ENGINE_LEVEL) {
     // the configuration engine when it takes the model and it fits a job
-    rc = mc::cfg_prepare(*desc, S->opt, req.cm);
     // A server without pruning keeps the block units for levels wider than a
     // warp: its exhaustive searches are the long requests that others are
     // seen to join and overtake (C3 literal outlasts 2 ms on blocks, not as
     // waves); with pruning, the default, wave units answer every request.
-    req.cm.waves = S->opt.prune != 0;
+    rc = mc::cfg_prepare(*desc, S->opt, req.cm, S->opt.prune != 0, false);
     if (rc == MC_OK && (req.cm.ab > kJobUnits || mc::cfg_tables_bytes(req.cm) > kJobTables)) rc = MC_ERR_INVAL;
     if (rc == MC_OK) {
       req.cfg = true;

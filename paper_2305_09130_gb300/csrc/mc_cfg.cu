@@ -637,8 +637,8 @@ __device__ void warp_role(const CfgLaunch& A) {
     if (u >= n) return;
     const uint64_t code = A.wunits ? __ldg(A.wunits_rev ? A.wunits - u : A.wunits + u) : 0ull;
     const CfgPass& Q = A.wunits ? A.passes[code >> 32] : A.one;
-    // a configuration, or (wave units of a single model: Q.group holds the
-    // segments' length above the lanes per state) a segment of one
+    // a configuration, or (wave units: Q.group holds the segments' length
+    // above the lanes per state) a segment of one
     const uint32_t part = A.wunits ? (uint32_t)code : __ldg(Q.order + u);
     const uint32_t segment = Q.group >> 8;
     const uint32_t cfg = segment ? part & 0xFFFFFFu : part;
@@ -671,7 +671,7 @@ __device__ void warp_role(const CfgLaunch& A) {
       __threadfence();
       const uint32_t done = atomicAdd(&Q.ctrl->units_done, 1u) + 1;
       const uint32_t ab = Q.p.a * Q.p.b;
-      last = done == (segment ? (uint32_t)__ldg(Q.seg + ab + 1) : ab);  // (segments: their number follows the starts)
+      last = done == (segment ? (uint32_t)__ldg(Q.seg) : ab);  // (wave units keep no log: their number)
       if (last) __threadfence();
     }
     last = __shfl_sync(0xffffffffu, last, 0);

@@ -34,7 +34,7 @@ uint64_t al256(uint64_t x) { return (x + 255) & ~255ull; }
 
 }  // namespace
 
-int cfg_prepare(const mc_model_desc& d_in, const mc_options& o, CfgModelPrep& M) {
+int cfg_prepare(const mc_model_desc& d_in, const mc_options& o, CfgModelPrep& M, bool waves, bool split) {
   mc_model_desc d = d_in;
   d.key_bits = 128;
   mc_options co = o;
@@ -69,6 +69,22 @@ int cfg_prepare(const mc_model_desc& d_in, const mc_options& o, CfgModelPrep& M)
   for (uint32_t k = 0; k < M.ab; ++k) M.order[k] = k;
   const uint32_t* N = M.params.data();
   std::stable_sort(M.order.begin(), M.order.end(), [N](uint32_t x, uint32_t y) { return N[x] > N[y]; });
+  M.waves = waves;
+  M.segment = 0;
+  M.units = M.ab;
+  if (split && waves && wave_model(M.p.rule, M.p.P, o.unit_threads)) {
+    uint32_t n_max = 0;
+    for (uint32_t k = 0; k < M.ab; ++k) n_max = std::max(n_max, N[k]);
+    for (uint32_t length = wave_segment(n_max, kWaveRunSegment); length && length < n_max; length *= 2) {
+      uint64_t units = 0;
+      for (uint32_t k = 0; k < M.ab; ++k) units += wave_segments(N[k], length);
+      if (units > M.ab + kRunExtraUnits) continue;
+      M.segment = length;
+      M.units = units;
+      M.seg[0] = units;  // (wave units keep no log)
+      break;
+    }
+  }
   // threads a block needs for this model's widest level in one round
   uint32_t t = 64;
   while ((uint64_t)t < M.unit_width * M.group && t < kCfgMaxThreads) t <<= 1;
@@ -187,12 +203,24 @@ void CfgRun::layout(uint32_t n_max, uint64_t units_max, uint8_t* dev, uint8_t* h
 
 void CfgRun::order_units(const std::vector<CfgModelPrep*>& models, const mc_options& opt) {
   order.clear();
+  full.clear();
   for (uint32_t k = 0; k < (uint32_t)models.size(); ++k) {
     const CfgModelPrep& M = *models[k];
     const uint32_t warp = cfg_warp_model(M, opt);
-    for (uint32_t c : M.order) order.push_back({M.params[c], k, c, warp});  // (params begin with N)
+    for (uint32_t c : M.order) {
+      const uint32_t n = M.params[c];  // (params begin with N)
+      const uint32_t length = M.segment ? M.segment : n;
+      for (uint32_t k0 = 0, part = 0; k0 < n; k0 += length, ++part) {
+        const uint32_t here = std::min(n - k0, length);
+        (M.segment && here == kWaveRunSegment ? full : order).push_back({here, k, part << 24 | c, warp});
+      }
+    }
   }
-  std::stable_sort(order.begin(), order.end(), [](const Unit& x, const Unit& y) { return x.n > y.n; });
+  // (full segments, most of a deep run's units, have their place: not sorted)
+  auto deeper = [](const Unit& x, const Unit& y) { return x.n > y.n; };
+  std::stable_sort(order.begin(), order.end(), deeper);
+  order.insert(std::upper_bound(order.begin(), order.end(), Unit{kWaveRunSegment, 0, 0, 0}, deeper), full.begin(),
+               full.end());
 }
 
 void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* queries, const mc_options& opt) {
@@ -222,7 +250,7 @@ void CfgRun::prepare(const std::vector<CfgModelPrep*>& models, const mc_query* q
       std::memset(&Q, 0, sizeof(Q));
       Q.p = M.p;
       Q.prune = opt.prune;
-      Q.group = M.group;
+      Q.group = M.group | M.segment << 8;
       Q.log_keys = M.d_keys;
       Q.log_par = M.d_par;
       Q.seg = M.d_seg;

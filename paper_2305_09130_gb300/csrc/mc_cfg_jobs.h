@@ -19,8 +19,10 @@ struct CfgModelPrep {
   uint32_t group = 1, ab = 0, L2 = 0, threads = 64, wcap = 32;
   uint64_t unit_width = 0, unit_log = 0, region = 0;
   bool waves = true;             // wave units allowed (mc_cfg_wave.h)
+  uint32_t segment = 0;          // their segments' length (0: configurations whole)
+  uint64_t units = 0;            // units of a pass: configurations or their segments
   std::vector<uint32_t> params;  // N, cost, speed
-  std::vector<uint64_t> seg;     // [ab + 1]
+  std::vector<uint64_t> seg;     // [ab + 1] ([0]: the units of a pass where configurations are split)
   std::vector<uint32_t> order;   // configurations, deepest first
   std::vector<uint32_t> wg, ts;  // values echoed in results
   uint8_t* base = nullptr;
@@ -34,7 +36,10 @@ struct CfgModelPrep {
 
 // Validate the description and lay the model out (host only).  Errors: as
 // mc_model_create, INVAL when the configuration engine cannot take it.
-int cfg_prepare(const mc_model_desc& d, const mc_options& o, CfgModelPrep& M);
+int cfg_prepare(const mc_model_desc& d, const mc_options& o, CfgModelPrep& M, bool waves = true, bool split = true);
+// Segments (split) add at most this many units to a model's configurations
+// (longer segments, where they would add more): 24 bytes each in a run's block.
+constexpr uint64_t kRunExtraUnits = 4096;
 // One warp per configuration: the options leave the block's threads to the
 // library, and the model takes wave units or its widest level's lanes fit a
 // warp.
@@ -78,9 +83,9 @@ struct CfgRun {
   // the (model, configuration) units, deepest first: made by order_units,
   // kept while the models stay the same (a batch's runs)
   struct Unit {
-    uint32_t n, model, cfg, warp;
+    uint32_t n, model, cfg, warp;  // (cfg: segment number << 24 | configuration where split)
   };
-  std::vector<Unit> order;
+  std::vector<Unit> order, full;
 
   uint64_t tables_cap = 0, tables_used = 0;     // model tables carried by the upload
   uint8_t *d_tables = nullptr, *h_tables = nullptr;

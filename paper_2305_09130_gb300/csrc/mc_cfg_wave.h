@@ -28,14 +28,18 @@ inline bool wave_model(uint32_t rule, uint32_t P, uint32_t unit_threads) {
 // explored by a warp of its own: the state in which every wave before an
 // instant has run is known (see mc_cfg_wave.cuh), so segments need not wait
 // for each other.  C3 literal's configurations of 4,096 work-groups are 32
-// warps instead of one.  (Runs of many models have warps enough and take a
-// configuration whole.)
+// warps instead of one.  A batch has more warps to begin with and pays for a
+// unit on the host too, so its segments are longer (256 models: 1,010 us a run
+// with configurations whole, 820 in segments of 512); a job of the request
+// loop takes configurations whole (its units are listed while requests wait:
+// 48 C3 requests take 1,060 us, and 1,070 in segments).
 constexpr uint32_t kWaveSegment = 128;
+constexpr uint32_t kWaveRunSegment = 512;
 
-inline uint32_t wave_segment(uint32_t n_max) {
+inline uint32_t wave_segment(uint32_t n_max, uint32_t length = kWaveSegment) {
   if (n_max >= 1u << 27) return 0;  // (the search for a segment's start sums starts in 32 bits)
   const uint32_t least = (uint32_t)(((uint64_t)n_max + 254) / 255);
-  return least > kWaveSegment ? least : kWaveSegment;
+  return least > length ? least : length;
 }
 inline uint64_t wave_segments(uint32_t n, uint32_t segment) { return ((uint64_t)n + segment - 1) / segment; }
 

@@ -138,3 +138,38 @@ def test_wave_units_match_oracle_and_blocks(mc, oracle, spec):
                 {k: exp[k] for k in ("t_min", "t_ini", "states", "checks", "i", "j", "level")}
             assert RP.decode(lay, r["witness_key"])[2] == exp["n"]
             RP.replay(spec, lay, r["trace"], lambda t: t == r["t_min"])
+
+
+def run_models():
+    """Models of a run: configurations of one and of several segments (512
+    work-groups), waves on their borders; a FREE model and an 11-unit one
+    beside them."""
+    out = []
+    for P, speed, N in ((6, [2] * 6, [1537, 512, 513, 5]), (5, [1, 2, 2, 3, 3], [1300, 1024, 40, 511]),
+                        (2, [2, 3], [2048, 700, 512, 1])):
+        deep = W.random_small(7420 + P, P, 2, 2, max(N), cost_max=5, rule=W.GREEDY, key_bits=128)
+        deep.speed, deep.n_workgroups = speed, N
+        out.append(deep)
+    out.append(W.random_small(7430, 3, 2, 2, 9, cost_max=5, speed_max=2, key_bits=128))
+    out.append(W.random_small(7431, 11, 2, 2, 9, cost_max=5, speed_max=2, rule=W.GREEDY, key_bits=128))
+    return out
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prune", (1, 0))
+def test_runs_in_segments_match_single_models(mc, prune):
+    specs = run_models()
+    opt = mc.mc_options_default(engine="config", prune=prune, search="single")
+    models = [mc.mc_model_create(s, opt) for s in specs]
+    mins = [mc.mc_min_time(m) for m in models]
+    batch = mc.mc_batch_create(specs, mc.mc_options_default(prune=prune))
+    for shift in (None, -1, 0, 1):
+        queries = [("min_time", None) if shift is None else ("check", m["t_min"] + shift) for m in mins]
+        for k, (r, m, q) in enumerate(zip(mc.mc_batch_run(batch, queries), models, queries)):
+            exp = mins[k] if shift is None else mc.mc_check(m, q[1])
+            assert (r["status"], r["states"]) == (0, exp["states"])
+            if shift is None or not exp["holds"]:
+                time, key = ("t_min", "witness_key") if shift is None else ("cex_time", "cex_key")
+                assert (r["time"], r["key"]) == (exp[time], exp[key])
+                assert mc.mc_batch_trace(batch, k) == exp["trace"]
+    mc.mc_batch_destroy(batch)
