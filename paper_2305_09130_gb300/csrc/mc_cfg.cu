@@ -1,4 +1,4 @@
-// Configuration engine: one thread block per (WG, TS) configuration.
+// Configuration engine: a thread block, or warps, per (WG, TS) configuration.
 //
 // After the two selects of `main` (Listing 3) every state carries the
 // configuration (i, j) it was selected with, and no transition changes it
@@ -30,11 +30,14 @@
 //     publishes the least violating time for a chained pass.
 //
 // Shared memory of a block: two frontiers (the level being expanded and the
-// next) of `wcap` keys and two open-addressing tables of `tsize` slots (the
-// next level's, and the one cleared for the level after it).  A slot is
-// claimed with a compare-and-swap from 0 (128-bit keys: atom.shared.cas.b128)
-// so two lanes inserting the same key meet at the same slot; a key is never
-// 0 (the WG index field is at least 1).
+// next) of `wcap` keys and, for GREEDY, two open-addressing tables of `tsize`
+// slots (the next level's, and the one cleared for the level after it).  A
+// slot is claimed with a compare-and-swap from 0 (128-bit keys:
+// atom.shared.cas.b128) so two lanes inserting the same key meet at the same
+// slot; a key is never 0 (the WG index field is at least 1).  FREE units
+// propose each state once (unit c only when no unit after c has started) and
+// use no table.  GREEDY models of up to ten units are explored by warps
+// (mc_cfg_wave.cuh), as are FREE levels that fit one.
 #include <cstdint>
 
 #include "mc_cfg_wave.h"
@@ -166,7 +169,7 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
   const uint32_t c_shift = (P - 1 - (unit_ok ? c : 0)) * n_bits;
   const K one_c = (K)1 << c_shift;
   const K after_c = one_c - 1;  // the count fields of the units after c
-  const bool log_on = Q.want_witness != 0;
+  const bool log_on = greedy && Q.want_witness != 0;  // (FREE: free_trace gives the path)
   const uint64_t seg0 = log_on ? Q.seg[cfg] : 0, seg1 = log_on ? Q.seg[cfg + 1] : 0;
   const uint32_t tmask = tsize - 1;
   const K key2 = ((K)(i + 1) << Q.p.wg_shift) | ((K)(j + 1) << Q.p.ts_shift);
@@ -306,8 +309,7 @@ __device__ void explore_unit(const CfgPass& Q, uint32_t cfg, uint64_t T, K* fron
 // s of the level is held by lanes [s*g, s*g + g), a unit starts only when no
 // later one has started, so a state is proposed once (mc_tree.cu), and the
 // proposals, ranked by a ballot, become the next level.  No table, no shared counter, no
-// block barrier; the same counts, records, log entries and early exit as
-// explore_unit.
+// block barrier; the same counts, records and early exit as explore_unit.
 
 // Position of set bit number k (from 0) of m; k < popc(m).
 __device__ __forceinline__ uint32_t nth_set_bit(uint32_t m, uint32_t k) {
@@ -355,8 +357,6 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
   const bool prune = Q.prune != 0, early = Q.early_exit != 0;
   const uint32_t* costp = Q.p.cost;
   const uint32_t* speedp = Q.p.speed;
-  void* const log_keys = Q.log_keys;
-  uint32_t* const log_par = Q.log_par;
   uint64_t* const levels = Q.levels;
   Ctrl* const ctrl = Q.ctrl;
   const uint32_t lane = threadIdx.x & 31u;
@@ -372,16 +372,8 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
   const uint32_t c_shift = (P - 1 - (unit_ok ? c : 0)) * n_bits;
   const K one_c = (K)1 << c_shift;
   const K after_c = one_c - 1;  // the count fields of the units after c
-  const bool log_on = Q.want_witness != 0;
-  const uint64_t seg0 = log_on ? Q.seg[cfg] : 0, seg1 = log_on ? Q.seg[cfg + 1] : 0;
-  const K key2 = ((K)(i + 1) << Q.p.wg_shift) | ((K)(j + 1) << Q.p.ts_shift);
-  if (log_on && lane == 0) {
-    log_store<K>(log_keys, seg0, key2);
-    log_par[seg0] = kNoParent;
-  }
-  K key = key2;  // the state of this lane's group (valid for my < W)
-  uint64_t lvl_base = seg0;
-  uint32_t W = 1, L = 2, deepest = 2, err = 0;
+  K key = ((K)(i + 1) << Q.p.wg_shift) | ((K)(j + 1) << Q.p.ts_shift);  // the state of this lane's group (valid for my < W)
+  uint32_t W = 1, L = 2, deepest = 2;
   uint32_t cut = kNoLevel;  // least level known to violate, read one level before it is used
   uint64_t vmin = kNone;
   while (L < 2 + N) {
@@ -401,39 +393,22 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
     const bool won = ok && (key & after_c) == 0;
     const uint32_t wm = __ballot_sync(0xffffffffu, won);
     const uint32_t Wn = __popc(wm);
-    if (won && log_on) {
-      const uint64_t at = lvl_base + W + __popc(wm & ((1u << lane) - 1u));
-      if (at < seg1) {
-        log_store<K>(log_keys, at, succ);
-        log_par[at] = (uint32_t)(lvl_base + my);
-      } else {
-        err = (uint32_t)MC_ERR_FRONTIER;
-      }
-    }
     // Step 2: a terminal winner with time <= T violates G(FIN -> time > T)
     if (L + 1 == 2 + N) vmin = warp_min_u64((won && (uint64_t)st <= T) ? (uint64_t)st : kNone);
-    if (Wn > spw) {  // cannot happen when the width bound holds
-      err = (uint32_t)MC_ERR_FRONTIER;
-      break;
-    }
+    if (Wn > spw) return (uint32_t)MC_ERR_FRONTIER;  // cannot happen when the width bound holds
     if (lane == 0 && Wn) atomicAdd(reinterpret_cast<unsigned long long*>(levels + 2 * (L + 1)), (unsigned long long)Wn);
     // the next level: state r from winner number r
     const uint32_t r = my < Wn ? my : 0u;
     key = shfl_key<K>(succ, Wn ? nth_set_bit(wm, r) : 0u);
     cut = sc ? ~sc : kNoLevel;
-    lvl_base += W;
     W = Wn;
     ++L;
     if (W == 0) break;
     deepest = L;
   }
-  // (uniform: the break above and a lane's log overflow)
-  const uint32_t errs = __ballot_sync(0xffffffffu, err != 0);
-  if (errs) return __shfl_sync(0xffffffffu, err, __ffs(errs) - 1);
   // this configuration's violating terminals (all at level 2 + N, held by
-  // the warp): the smallest key of the least time, and its log index
+  // the warp): the smallest key of the least time
   uint64_t whi = kNone, wlo = kNone;
-  uint32_t widx = 0;
   if (vmin != kNone) {
     if (lane == 0 && early) atomicMax(&ctrl->stop_c, ~(2u + N));
     const bool mine = my < W && c == 0;
@@ -450,19 +425,168 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
     whi = warp_min_u64(cand ? (uint64_t)KeyOps<K>::hi(key) : kNone);
     const bool cand_hi = cand && (uint64_t)KeyOps<K>::hi(key) == whi;
     wlo = warp_min_u64(cand_hi ? (uint64_t)KeyOps<K>::lo(key) : kNone);
-    const uint32_t wl = __ballot_sync(0xffffffffu, cand_hi && (uint64_t)KeyOps<K>::lo(key) == wlo);
-    widx = (uint32_t)(lvl_base + (uint32_t)(__ffs(wl) - 1) / g);
   }
   if (lane == 0) {
     CfgRec rec;
     rec.vpack = vmin != kNone ? pack_tij(vmin, i, j) : kNone;
     rec.wkey_lo = vmin != kNone ? wlo : kNone;
     rec.wkey_hi = vmin != kNone ? whi : kNone;
-    rec.widx = vmin != kNone ? widx : 0u;
+    rec.widx = 0;
     rec.deepest = deepest;
     Q.rec[cfg] = rec;
   }
   return 0;
+}
+
+// ------------------------------------------------------------------ chain units
+// FREE configurations of 2 to 4 units, a block each.  Under FREE a state is
+// any choice of work-group counts with a sum of at most N and, when pruning,
+// every unit's clock within T (clocks only grow, so every state on the way is
+// kept too).  In the order in which later units start last (above), the
+// states that share the counts of all units but the last form a chain, one
+// state per level, which needs nothing from other chains.  So a thread takes
+// chains and walks them, with no barrier and no frontier; the states are
+// counted by level in shared memory.
+//
+// What bounds it: the longest chain, a few instructions per state, and the
+// search for chains: a thread finds its next one among all counts up to N,
+// of which 1 in (P-1)! is one (sums above N), so five units and more stay
+// with explore_unit, whose configurations are at most a dozen levels deep
+// there.  Measured: a C1 min-time query (P = 2, 64 work-groups, three passes)
+// 106 us with explore_unit and its trace walked through the log, 64 us here
+// with the trace built from the witness's counts (free_trace).
+constexpr uint32_t kChainMaxP = 4;
+
+__device__ __forceinline__ bool chain_unit(const Params& p) {
+  return p.rule == MC_FREE && p.P >= 2 && p.P <= kChainMaxP;
+}
+
+template <class K, class C>
+__device__ void explore_chains(const CfgPass& Q, uint32_t cfg, uint64_t T, uint32_t* hist, CfgShared& S) {
+  const uint32_t tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31u;
+  const uint32_t P = Q.p.P, n_bits = Q.p.n_bits, b = Q.p.b, head = P - 1;
+  const bool early = Q.early_exit != 0;
+  const uint32_t i = cfg / b, j = cfg % b;
+  const uint32_t N = __ldg(Q.p.N + cfg);
+  Ctrl* const ctrl = Q.ctrl;
+  const C Tc = Q.prune && T < (uint64_t)(C)~(C)0 ? (C)T : (C)~(C)0;
+  // the units' times and the most work-groups each may take
+  C t[kChainMaxP];
+  uint32_t most[kChainMaxP];
+#pragma unroll
+  for (uint32_t u = 0; u < kChainMaxP; ++u) {
+    t[u] = u < P ? (C)((uint64_t)__ldg(Q.p.cost + cfg) * __ldg(Q.p.speed + u)) : (C)1;
+    const C q = Tc / t[u];
+    most[u] = u >= P ? 0u : q < (C)N ? (uint32_t)q : N;
+  }
+  C t_last = t[1];
+  uint32_t most_last = most[1];
+#pragma unroll
+  for (uint32_t u = 2; u < kChainMaxP; ++u)
+    if (u == head) {
+      t_last = t[u];
+      most_last = most[u];
+    }
+  const uint32_t d1 = head > 1 ? most[1] + 1 : 1, d2 = head > 2 ? most[2] + 1 : 1;
+  const uint32_t chains = (most[0] + 1) * d1 * d2;
+  for (uint32_t x = tid; x <= N; x += nthr) hist[x] = 0;
+  __syncthreads();
+  const K key2 = ((K)(i + 1) << Q.p.wg_shift) | ((K)(j + 1) << Q.p.ts_shift);
+  uint64_t best = kNone;
+  K best_key = 0;
+  // early exit: the least level known to violate, asked for every eighth chain
+  uint32_t cut = kNoLevel, round = 0;
+  for (uint32_t x = tid; x < chains; x += nthr, ++round) {
+    if (early && (round & 7u) == 0) {
+      const uint32_t sc = ld_relaxed_u32(&ctrl->stop_c);
+      if (sc) cut = ~sc;
+    }
+    const uint32_t x1 = x / d2, n2 = x - x1 * d2;
+    const uint32_t n0 = x1 / d1, n1 = x1 - n0 * d1;
+    const uint32_t taken = n0 + n1 + n2;
+    if (taken > N || 2 + taken > cut) continue;
+    C mx = (C)n0 * t[0];
+    K key = key2 | ((K)n0 << (head * n_bits));
+    if (head > 1) {
+      const C f = (C)n1 * t[1];
+      mx = f > mx ? f : mx;
+      key |= (K)n1 << ((head - 1) * n_bits);
+    }
+    if (head > 2) {
+      const C f = (C)n2 * t[2];
+      mx = f > mx ? f : mx;
+      key |= (K)n2 << n_bits;
+    }
+    const uint32_t end = min(min(N, taken + most_last), cut - 2);  // (levels beyond the cut are not counted)
+    for (uint32_t k = taken; k <= end; ++k) atomicAdd(hist + k, 1u);
+    if (end == N) {  // Step 2: a terminal with time <= T violates G(FIN -> time > T)
+      const C last = (C)(N - taken) * t_last;
+      const uint64_t time = (uint64_t)(last > mx ? last : mx);
+      key |= (K)(N - taken);
+      if (time <= T && (time < best || (time == best && key < best_key))) {
+        best = time;
+        best_key = key;
+      }
+    }
+  }
+  const uint64_t wb = warp_min_u64(best);
+  if (lane == 0 && wb != kNone) atomicMin(&S.vmin, (unsigned long long)wb);
+  __syncthreads();
+  // the widths; the smallest key of the least time
+  const uint64_t tv = S.vmin;
+  if (tid == 0 && early && tv != kNone) atomicMax(&ctrl->stop_c, ~(2u + N));
+  uint32_t deep = 0;
+  for (uint32_t k = 1 + tid; k <= N; k += nthr) {
+    const uint32_t w = hist[k];
+    if (!w) continue;
+    atomicAdd(reinterpret_cast<unsigned long long*>(Q.levels + 2ull * (2 + k)), (unsigned long long)w);
+    deep = k;
+  }
+  deep = __reduce_max_sync(0xffffffffu, deep);
+  if (lane == 0 && deep) atomicMax(&S.widx, deep);
+  const bool mine = tv != kNone && best == tv;
+  const uint64_t whi = warp_min_u64(mine ? (uint64_t)KeyOps<K>::hi(best_key) : kNone);
+  if (lane == 0 && whi != kNone) atomicMin(&S.whi, (unsigned long long)whi);
+  __syncthreads();
+  const uint64_t wlo = warp_min_u64(mine && (uint64_t)KeyOps<K>::hi(best_key) == S.whi ? (uint64_t)KeyOps<K>::lo(best_key) : kNone);
+  if (lane == 0 && wlo != kNone) atomicMin(&S.wlo, (unsigned long long)wlo);
+  __syncthreads();
+  if (tid == 0) {
+    CfgRec rec;
+    rec.vpack = tv != kNone ? pack_tij(tv, i, j) : kNone;
+    rec.wkey_lo = tv != kNone ? S.wlo : kNone;
+    rec.wkey_hi = tv != kNone ? S.whi : kNone;
+    rec.widx = 0;
+    rec.deepest = 2 + S.widx;
+    Q.rec[cfg] = rec;
+  }
+}
+
+// The trace s0 -> the witness of a FREE pass's configuration (i, j): the path
+// in the order in which the states were generated (all of a unit's
+// work-groups before the next unit's), a level per thread.  No clock on the
+// way passes the witness's time, so each state was explored.
+template <class K>
+__device__ void free_trace(const CfgPass& Q, uint32_t i, uint32_t j, uint32_t stop, uint32_t first, uint32_t step) {
+  const Params& p = Q.p;
+  const CfgRec* r = Q.rec + (uint64_t)i * p.b + j;
+  K key = (K)__ldcg(&r->wkey_lo);
+  if (sizeof(K) == 16) key |= (K)((u128)__ldcg(&r->wkey_hi) << 64);
+  const K k1 = (K)(i + 1) << p.wg_shift;
+  for (uint32_t l = first; l <= stop; l += step) {
+    K k = l == 0 ? (K)0 : k1;
+    if (l >= 2) {
+      k |= (K)(j + 1) << p.ts_shift;
+      uint32_t rest = l - 2;
+      for (uint32_t u = 0; u < p.P; ++u) {
+        const uint32_t shift = (p.P - 1 - u) * p.n_bits, n = min(rest, (uint32_t)field(key, shift, p.n_mask));
+        k |= (K)n << shift;
+        rest -= n;
+      }
+    }
+    Q.trace[2 * l] = KeyOps<K>::lo(k);
+    Q.trace[2 * l + 1] = KeyOps<K>::hi(k);
+  }
 }
 
 }  // namespace
@@ -569,8 +693,13 @@ __device__ void cfg_epilogue(const CfgPass& Q, uint64_t T, CfgShared& S) {
   for (uint32_t l = 3 + tid; l <= last; l += nthr) part += __ldcg(Q.levels + 2 * l);
   atomicAdd(&S.e_sum, (unsigned long long)part);
   __syncthreads();
-  if (tid != 0) return;
-  epilogue_publish<K>(Q, T, stop, last, (uint64_t)S.e_best, (uint64_t)S.e_wpack, (uint64_t)S.e_sum, true);
+  const bool free = p.rule == MC_FREE;
+  if (tid == 0)
+    epilogue_publish<K>(Q, T, stop, last, (uint64_t)S.e_best, (uint64_t)S.e_wpack, (uint64_t)S.e_sum, !free);
+  if (free && Q.want_witness && stop != kNoLevel) {
+    const uint64_t w = S.e_wpack;
+    free_trace<K>(Q, pack_i(w), pack_j(w), stop, tid, nthr);
+  }
 }
 
 // The warp that finished a pass's last configuration, when it is a warp
@@ -613,7 +742,8 @@ __device__ void cfg_epilogue_warp(const CfgPass& Q, uint64_t T) {
   for (uint32_t l = 3 + lane; l <= last; l += 32) part += __ldcg(Q.levels + 2 * l);
   const uint64_t sum = warp_sum_u64(part);
   const bool wave = wave_unit(p);
-  if (lane == 0) epilogue_publish<K>(Q, T, stop, last, best, wpack, sum, !wave);
+  if (lane == 0) epilogue_publish<K>(Q, T, stop, last, best, wpack, sum, false);
+  if (!wave && Q.want_witness && stop != kNoLevel) free_trace<K>(Q, pack_i(wpack), pack_j(wpack), stop, lane, 32);
   if (wave && Q.want_witness && stop != kNoLevel) {
     const CfgRec* r = Q.rec + (uint64_t)pack_i(wpack) * p.b + pack_j(wpack);
     K key = (K)__ldcg(&r->wkey_lo);
@@ -750,7 +880,10 @@ __global__ void __launch_bounds__(kCfgMaxThreads) cfg_kernel(const __grid_consta
     __syncthreads();
     const uint64_t T = S.T;
     if (!S.skip) {
-      if (Q.p.clk32) explore_unit<K, uint32_t>(Q, cfg, T, front0, front1, tab0, tab1, A.wcap, A.tsize, S);
+      uint32_t* const hist = reinterpret_cast<uint32_t*>(front0);  // (at least wcap > N keys)
+      if (chain_unit(Q.p) && Q.p.clk32) explore_chains<K, uint32_t>(Q, cfg, T, hist, S);
+      else if (chain_unit(Q.p)) explore_chains<K, uint64_t>(Q, cfg, T, hist, S);
+      else if (Q.p.clk32) explore_unit<K, uint32_t>(Q, cfg, T, front0, front1, tab0, tab1, A.wcap, A.tsize, S);
       else explore_unit<K, uint64_t>(Q, cfg, T, front0, front1, tab0, tab1, A.wcap, A.tsize, S);
       __syncthreads();
       if (tid == 0 && S.err) set_error(Q.ctrl, (int)S.err);
