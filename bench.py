@@ -212,9 +212,8 @@ def algorithmic_bytes_per_state(P: int, key_words: int) -> int:
 
 def ordered_bytes_per_state(key_words: int) -> int:
     """Per unique state of the ordered pass, which keeps no visited set: its
-    key written to and read back from the frontier log, and its 4-byte parent
-    index."""
-    return 2 * 8 * key_words + 4
+    key written to and read back from the frontier log."""
+    return 2 * 8 * key_words
 
 
 def kernel_source_hash(srcs=KERNEL_SRCS) -> str:

@@ -13,21 +13,24 @@
 // A state that is generated once needs no visited set: no table is
 // allocated, cleared or probed.
 //
-// The frontier log with its parent indices, the level records, the level
-// barrier fused with the width counter and the tagged log entries are those of
-// the general pass.
+// The frontier log, the level records, the level barrier fused with the width
+// counter and the tagged log entries are those of the general pass.  The log's
+// parent indices are neither written nor read: a state's counts name its path
+// (all work-groups of unit 0, then unit 1's, ...), so the trace is built from
+// the witness, a level per thread, and the witness's place is not looked up.
 //
-// What bounds it: on wide levels the log, each key and parent index written
-// once and each key read once by the next level (36 bytes a state with
-// 128-bit keys: C3 at G=36 moves 5.2 TB/s of the 6.8 TB/s a copy reaches, the
-// rest waits at the tiles' barriers); on narrow ones the chain of a level (key
-// load, reservation fused with the arrival, poll; 3.4 us a level on C2 at
-// G=80).  A tile is blockDim x R keys, R up to kTreeKeys, so that one
-// reservation (an atomic on the level's one word) covers a thousand states; the
-// next tile's keys are loaded before the reservation is waited for.  In a level
-// with fewer states than threads a tile is one key per thread.  Measured on C3
-// at G=28: 4 keys per thread and 4 blocks of 256 per SM 1.37 ms, 2 blocks of
-// 512 1.39, 8 of 128 1.40; 6 keys spill, 6 blocks (40 registers) 1.87.
+// What bounds it: on wide levels the log, each key written once and read once
+// by the next level (32 bytes a state with 128-bit keys: C3 at G=36 moves 5.1
+// of the 6.8 TB/s a copy reaches, the rest waits at the tiles' barriers; a
+// query takes 6.85 ms, and took 7.14 with parent indices written, 36 bytes);
+// on narrow ones the chain of a level (key load, reservation fused with the
+// arrival, poll; 3.4 us a level on C2 at G=80).  A tile is blockDim x R keys,
+// R up to kTreeKeys, so that one reservation (an atomic on the level's one
+// word) covers a thousand states; the next tile's keys are loaded before the
+// reservation is waited for.  In a level with fewer states than threads a
+// tile is one key per thread.  Measured on C3 at G=28 (with parent indices):
+// 4 keys per thread and 4 blocks of 256 per SM 1.37 ms, 2 blocks of 512 1.39,
+// 8 of 128 1.40; 6 keys spill, 6 blocks (40 registers) 1.87.
 #include "mc_explore.cuh"
 #include "mc_tree.h"
 
@@ -233,7 +236,6 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
         key = ((A)(y / p.b + 1) << p.wg_shift) | ((A)(y % p.b + 1) << p.ts_shift);
       }
       KeyOps<K>::store(G.log_keys, x, log.pack(key));
-      G.log_par[x] = x == 0 ? kNoParent : x <= p.a ? 0u : (uint32_t)((x - 1 - p.a) / p.b);
     }
     if (gtid == 0) {
       ctrl->T = T;
@@ -322,7 +324,6 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
       }
       // the next tile's keys are on their way while this tile's places are
       // reserved and its successors written
-      const uint32_t here = base;
       base += stride;
       if (more) {
 #pragma unroll
@@ -353,15 +354,10 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
         const uint64_t at0 = offN + s_base + before;
         if (at0 + wcnt <= G.log_cap) {
           K* const dst = reinterpret_cast<K*>(G.log_keys) + at0;
-          uint32_t* const par = G.log_par + at0;
           const uint32_t below = (1u << lane) - 1u;
-          auto put = [&](uint32_t& at, bool mine, A succ, uint32_t parent) {  // a warp's stores are consecutive
+          auto put = [&](uint32_t& at, bool mine, A succ) {  // a warp's stores are consecutive
             const uint32_t m = __ballot_sync(0xffffffffu, mine);
-            if (mine) {
-              const uint32_t to = at + __popc(m & below);
-              LogIO<K>::store(dst, to, log.pack(succ), lpol);
-              st_u32_ef(par + to, parent, lpol);
-            }
+            if (mine) LogIO<K>::store(dst, at + __popc(m & below), log.pack(succ), lpol);
             at += __popc(m);
           };
           // the last unit's successors first, the others behind them: rows
@@ -370,17 +366,16 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
 #pragma unroll
           for (int r = 0; r < kTreeKeys; ++r) {
             if (r >= (int)R) continue;
-            const uint32_t s = here + r * blockDim.x;
             if (PRUNE) {
               for (uint32_t any = __reduce_or_sync(0xffffffffu, starts[r]); any; any &= any - 1) {
                 const uint32_t f = __ffs(any) - 1;
-                put(at, (starts[r] >> f) & 1u, key[r] + ((A)1 << (f * p.n_bits)), s);
+                put(at, (starts[r] >> f) & 1u, key[r] + ((A)1 << (f * p.n_bits)));
               }
             } else {
-              put(at, starts[r] != 0, key[r] + 1, s);
+              put(at, starts[r] != 0, key[r] + 1);
               A one = (A)1 << p.n_bits;
               for (uint32_t f = 1; __any_sync(0xffffffffu, f < starts[r]); ++f, one <<= p.n_bits)
-                put(other, f < starts[r], key[r] + one, s);
+                put(other, f < starts[r], key[r] + one);
             }
           }
         } else if (lane == 0) {  // beyond the log's capacity: nothing is written, the query fails
@@ -478,36 +473,30 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
     }
     if (!grid_sync(bar, epoch)) return;
   }
-  {
-    const uint64_t lo = ld_relaxed_u64(&ctrl->wkey_lo), hi = sizeof(A) == 16 ? ld_relaxed_u64(&ctrl->wkey_hi) : 0;
-    for (uint64_t x = gtid; x < Ww; x += nthreads) {
-      A key;
-      if (!tree_entry(G, log, offW + x, KeyOps<K>::load(G.log_keys, offW + x), key)) break;
-      if (KeyOps<A>::lo(key) == lo && KeyOps<A>::hi(key) == hi) ctrl->widx = x;
-    }
+  // the trace s0 -> the witness, in the order in which states are generated
+  if (blockIdx.x) return;
+  const uint64_t lo = ld_relaxed_u64(&ctrl->wkey_lo), hi = sizeof(A) == 16 ? ld_relaxed_u64(&ctrl->wkey_hi) : 0;
+  if (lo == kNone || (sizeof(A) == 16 && hi == kNone)) {  // cannot happen when the level is intact
+    if (tid == 0) set_error(ctrl, MC_ERR_FRONTIER);
+    return;
   }
-  if (!grid_sync(bar, epoch)) return;
-  // trace: follow parent indices from the witness back to s0
-  if (gtid == 0) {
+  const A witness = sizeof(A) == 16 ? (A)(((u128)hi << 64) | lo) : (A)lo;
+  for (uint32_t l = tid; l <= wl; l += blockDim.x) {
+    A key = l >= 1 ? (A)(ti + 1) << p.wg_shift : (A)0;
+    if (l >= 2) {
+      key |= (A)(tj + 1) << p.ts_shift;
+      uint32_t rest = l - 2;
+      for (uint32_t u = 0; u < p.P; ++u) {
+        const uint32_t shift = (p.P - 1 - u) * p.n_bits, n = min(rest, (uint32_t)field(witness, shift, p.n_mask));
+        key |= (A)n << shift;
+        rest -= n;
+      }
+    }
+    G.trace[2 * l] = KeyOps<A>::lo(key);
+    G.trace[2 * l + 1] = KeyOps<A>::hi(key);
+  }
+  if (tid == 0) {
     if (sizeof(A) == 8) ctrl->wkey_hi = 0;
-    uint64_t idx = ld_relaxed_u64(&ctrl->widx);
-    if (idx >= Ww) {  // cannot happen when the level is intact; never walk from it
-      set_error(ctrl, MC_ERR_FRONTIER);
-      return;
-    }
-    uint64_t off = offW;
-    for (uint32_t l = wl;; --l) {
-      const uint64_t at = off + idx;
-      const K raw = KeyOps<K>::load(G.log_keys, at);
-      const uint32_t par = __ldcg(G.log_par + at);
-      if (l) off = ld_relaxed_u64(&G.off[l - 1]);  // in flight together
-      A key;
-      if (!tree_entry(G, log, at, raw, key)) return;
-      G.trace[2 * l] = KeyOps<A>::lo(key);
-      G.trace[2 * l + 1] = KeyOps<A>::hi(key);
-      if (l == 0) break;
-      idx = par;
-    }
     ctrl->witness_level = wl;
     ctrl->trace_len = wl + 1;
   }
