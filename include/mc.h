@@ -119,14 +119,15 @@ typedef enum {
                             with 128-bit keys), else LEVEL                    */
   MC_ENGINE_LEVEL = 1,   /* level-synchronous BFS over the whole state space:
                             one persistent cooperative launch per pass, a
-                            device-wide barrier per level, the visited set in
-                            device memory (any model)                         */
-  MC_ENGINE_CONFIG = 2   /* one thread block per (WG, TS) configuration: the
-                            selects of Listing 3 split the states below level 2
-                            into disjoint subtrees, and a block explores one
-                            subtree with its frontier and visited set in shared
-                            memory and a block-wide barrier per level (models
-                            whose per-configuration levels fit, see AUTO)     */
+                            device-wide barrier per level, the visited set (if
+                            any, see mc_probe_scheme) in device memory (any
+                            model)                                            */
+  MC_ENGINE_CONFIG = 2   /* the (WG, TS) configurations apart: the selects of
+                            Listing 3 split the states below level 2 into
+                            disjoint subtrees, and a warp or a thread block
+                            explores one subtree, or a part of one, in
+                            registers and shared memory (models whose
+                            per-configuration levels fit, see AUTO)           */
 } mc_engine;
 
 typedef struct mc_model mc_model;

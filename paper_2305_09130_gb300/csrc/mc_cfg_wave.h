@@ -13,10 +13,10 @@ namespace mc {
 // current instant: 2^P bits, one 32-bit word per lane, so 2^10 subsets fill
 // the warp.  (Above, a level needs several words per lane and the block
 // units' hashed tables take over.)  Faster than the block units at every P:
-// counts of 60 configurations, one speed, 4,096 work-groups take 0.24 ms
-// against 3.4 ms (P = 1), 0.46 / 3.6 (2), 0.32 / 3.7 (4), 0.34 / 4.6 (8), and
-// of 1,024 work-groups 0.11 / 3.7 ms (10).  mc_options.unit_threads asks for
-// blocks.
+// counts of 60 configurations of 4,096 work-groups, each whole, one speed,
+// take 0.24 ms against 3.4 ms (P = 1), 0.46 / 3.6 (2), 0.32 / 3.7 (4),
+// 0.34 / 4.6 (8), and of 1,024 work-groups 0.11 / 3.7 ms (10).
+// mc_options.unit_threads asks for blocks.
 constexpr uint32_t kWaveMaxP = 10;
 
 inline bool wave_model(uint32_t rule, uint32_t P, uint32_t unit_threads) {
