@@ -125,10 +125,10 @@ __device__ __forceinline__ bool tree_entry(const ExploreArgs& G, const TreeLog<K
 // terminal (FIN, Listing 4), those within T violate G(FIN -> time > T) (Step
 // 2), and the least of them lowers `best`.  The units of the fields below f0
 // have not started, so their next clocks are one work-group each; `least[f]`
-// is the least speed of the fields below f.  Clocks in C: 32 bits when every
-// clock of the model fits.  (One state in five has terminal successors on C3
-// at G=36: with a loop per field and per successor in 64 bits this was 40% of
-// the pass.)
+// (f > 0) is the least speed of the fields below f.  Clocks in C: 32 bits when
+// every clock of the model fits.  (One state in five has terminal successors
+// on C3 at G=36: with a loop per field and per successor in 64 bits this was
+// 40% of the pass.)
 template <bool PRUNE, class C, class A>
 __device__ __forceinline__ void tree_times(const Params& p, A key, uint32_t f0, uint64_t cost, bool terminal,
                                            uint64_t T, uint32_t i, uint32_t j, const uint32_t* speed,
@@ -155,7 +155,9 @@ __device__ __forceinline__ void tree_times(const Params& p, A key, uint32_t f0, 
       if ((uint64_t)max(mx, (C)speed[f]) * cost > T) starts &= ~(1u << f);
   }
   if (terminal) {
-    const uint64_t t = (uint64_t)max(mx, min(own, (C)least[f0])) * cost;
+    // (no field below the lowest: only `own`, which 64-bit clocks may take
+    // beyond any 32-bit stand-in for "none")
+    const uint64_t t = (uint64_t)max(mx, f0 ? min(own, (C)least[f0]) : own) * cost;
     if (t <= T && t <= pack_time(best)) best = min(best, pack_tij(t, i, j));
   }
 }

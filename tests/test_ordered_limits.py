@@ -1,0 +1,49 @@
+"""Ordered expansion of FREE models at the limits of its arithmetic: clocks
+that exceed 32 bits by a unit's speed alone, compared with the oracle and with
+the pass that keeps a visited set."""
+import pytest
+
+import replay as RP
+from paper_2305_09130_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+NO_LIMIT = (1 << 64) - 1
+BIG = 1 << 31
+
+
+def fast_and_slow(speed, n, cost):
+    k = len(n)
+    return W.ModelSpec("speeds_" + "_".join(map(str, speed)), len(speed), [1], list(range(1, k + 1)), n, cost, speed)
+
+
+@pytest.mark.parametrize("spec", [fast_and_slow([BIG], [4, 3], [1, 2]),
+                                  fast_and_slow([1, 2 * BIG - 1], [5, 2, 9], [3, 1, 2]),
+                                  fast_and_slow([2 * BIG - 1, 1], [6, 3], [1, 4]),
+                                  fast_and_slow([2 * BIG - 1, 2 * BIG - 1], [3, 5], [1, 1]),
+                                  fast_and_slow([BIG, 7, BIG + 5], [4, 6], [2, 1]),
+                                  fast_and_slow([1 << 30, BIG - 1, BIG, 3, BIG + 1], [5, 4], [1, 1])],
+                         ids=lambda s: s.name)
+def test_speeds_beyond_32_bits_of_clock(mc, oracle, spec):
+    t_min = oracle.min_time(spec)["t_min"]
+    models = [mc.mc_model_create(spec, mc.mc_options_default(engine="level", **o)) for o in ({}, {"probe_scheme": "split"})]
+    lay = mc.mc_model_layout(models[0])
+    for T in (0, t_min - 1, t_min, (1 << 32) - 1, 1 << 32, 3 * BIG, 1 << 33, 1 << 34, NO_LIMIT):
+        for prune, ee in ((1, 1), (0, 1), (1, 0), (0, 0)):
+            exp = oracle.check(spec, T, prune=bool(prune), early_exit=bool(ee))
+            for m in models:
+                mc.mc_set_options(m, mc.mc_options_default(engine="level", prune=prune, early_exit=ee))
+                r = mc.mc_check(m, T)
+                assert (r["holds"], r["states"], r["levels"]) == (exp["holds"], exp["states"], exp["levels"])
+                if not exp["holds"]:
+                    i, j, n = RP.decode(lay, r["cex_key"])
+                    assert (r["cex_time"], i - 1, j - 1, r["cex_level"], n) == (
+                        exp["cex_time"], exp["cex_i"], exp["cex_j"], exp["cex_level"], exp["cex_n"])
+                    RP.replay(spec, lay, r["trace"], lambda t: t == r["cex_time"])
+    for search in ("single", "lower", "bisect"):
+        exp = oracle.min_time(spec, search=search)
+        for m in models:
+            mc.mc_set_options(m, mc.mc_options_default(engine="level", search=search))
+            r = mc.mc_min_time(m)
+            assert {k: r[k] for k in ("t_min", "t_ini", "states", "checks", "i", "j", "level")} == {
+                k: exp[k] for k in ("t_min", "t_ini", "states", "checks", "i", "j", "level")}
