@@ -62,30 +62,32 @@ __device__ __forceinline__ uint32_t lowest_bit<u128>(u128 x) {
 template <class K, class A>
 struct TreeLog;
 
-__device__ __forceinline__ bool strip_tag(uint64_t w, uint32_t tag_hi, uint32_t limit, uint64_t& key) {
+__device__ __forceinline__ bool strip_tag(uint64_t w, uint32_t tag_hi, uint32_t most, uint64_t& key) {
   const uint32_t hi = (uint32_t)(w >> 32) ^ tag_hi;
   key = ((uint64_t)hi << 32) | (uint32_t)w;
-  return hi < limit;
+  return hi <= most;
 }
 
 template <>
 struct TreeLog<uint64_t, uint64_t> {
-  uint32_t tag_hi, limit;  // the tag in a word's upper half; what that half of a key stays below
+  // the tag in a word's upper half; the most that half of a key can be (all
+  // ones without a tag: a key of 64 used bits may have them all set)
+  uint32_t tag_hi, most;
   __device__ TreeLog(uint32_t tb, uint64_t tag) : tag_hi(tb ? (uint32_t)tag << (32 - tb) : 0u),
-                                                  limit(tb ? 1u << (32 - tb) : 0xFFFFFFFFu) {}
+                                                  most(0xFFFFFFFFu >> tb) {}
   __device__ uint64_t pack(uint64_t k) const { return k | ((uint64_t)tag_hi << 32); }
-  __device__ bool unpack(uint64_t w, uint64_t& key) const { return strip_tag(w, tag_hi, limit, key); }
+  __device__ bool unpack(uint64_t w, uint64_t& key) const { return strip_tag(w, tag_hi, most, key); }
 };
 
 template <>
 struct TreeLog<u128, uint64_t> {
-  uint32_t tag_hi, limit;
+  uint32_t tag_hi, most;
   uint64_t high;
   __device__ TreeLog(uint32_t tb, uint64_t tag) : tag_hi(tb ? (uint32_t)tag << (32 - tb) : 0u),
-                                                  limit(tb ? 1u << (32 - tb) : 0xFFFFFFFFu), high(tb ? tag : 0) {}
+                                                  most(0xFFFFFFFFu >> tb), high(tb ? tag : 0) {}
   __device__ u128 pack(uint64_t k) const { return ((u128)high << 64) | k | ((uint64_t)tag_hi << 32); }
   __device__ bool unpack(u128 w, uint64_t& key) const {
-    return strip_tag((uint64_t)w, tag_hi, limit, key) && (uint64_t)(w >> 64) == high;
+    return strip_tag((uint64_t)w, tag_hi, most, key) && (uint64_t)(w >> 64) == high;
   }
 };
 

@@ -1,6 +1,6 @@
 """Ordered expansion of FREE models at the limits of its arithmetic: clocks
-that exceed 32 bits by a unit's speed alone, compared with the oracle and with
-the pass that keeps a visited set."""
+that exceed 32 bits by a unit's speed alone, and keys that fill their word,
+compared with the oracle and with the pass that keeps a visited set."""
 import pytest
 
 import replay as RP
@@ -47,3 +47,26 @@ def test_speeds_beyond_32_bits_of_clock(mc, oracle, spec):
             r = mc.mc_min_time(m)
             assert {k: r[k] for k in ("t_min", "t_ini", "states", "checks", "i", "j", "level")} == {
                 k: exp[k] for k in ("t_min", "t_ini", "states", "checks", "i", "j", "level")}
+
+
+def test_keys_that_fill_their_word(mc):
+    """64 used bits leave no room for a tag, and the upper half of a key is all
+    ones in the last configuration (1023, 511) from n_0 = 32764 on.  Pruning
+    keeps the other configurations and units from starting."""
+    a, b, N = 1023, 511, 32767
+    spec = W.ModelSpec("ones", 3, list(range(a)), list(range(b)), [1] * (a * b - 1) + [N],
+                       [N + 1] * (a * b - 1) + [1], [1, N + 1, N + 1])
+    got = []
+    for o in ({}, {"table_log2": 20}):
+        m = mc.mc_model_create(spec, mc.mc_options_default(engine="level", log_capacity=600_000,
+                                                           barrier_timeout_ns=2_000_000_000, **o))
+        lay = mc.mc_model_layout(m)
+        assert lay["used_bits"] == 64 and lay["log_tag_bits"] == 0
+        r = mc.mc_check(m, N)
+        assert r["cex_key"] >> 32 == 0xFFFFFFFF
+        assert (r["cex_time"], r["cex_i"], r["cex_j"], r["cex_level"]) == (N, a - 1, b - 1, 2 + N)
+        assert r["states"] == 1 + a + a * b + N
+        RP.replay(spec, lay, r["trace"], lambda t: t == N)
+        got.append({k: v for k, v in r.items() if k != "trace"})
+        mc.mc_model_destroy(m)
+    assert got[0] == got[1]
