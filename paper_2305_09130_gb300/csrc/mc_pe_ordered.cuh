@@ -328,6 +328,9 @@ __global__ void __launch_bounds__(kPeThreads, 2) pe_ordered_kernel(const __grid_
           solo.keys[0][x] = key;
         }
         __syncthreads();
+        // an entry that never appeared is not a key: nothing decodes it, the
+        // pass ends with the error that entry() set
+        if (s_flags & kPeFlagError) end = 1;
         while (!end) {
           const uint64_t offN = off + n;
           uint64_t best = kNone;

@@ -1,0 +1,37 @@
+"""Orders that the device code keeps and that no run can show broken without
+harm: read from the sources, with the arithmetic that makes them necessary
+restated here."""
+import os
+import re
+
+from conftest import ROOT
+
+CSRC = os.path.join(ROOT, "paper_2305_09130_gb300", "csrc")
+
+
+def source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def between(text, start, end):
+    at = text.index(start)
+    return text[at:text.index(end, at)]
+
+
+def test_narrow_levels_decode_only_entries_that_appeared():
+    """A log entry that does not appear within the wait limit leaves a raw word
+    behind.  Decoded, an untouched (zero) word names configuration -1 of -1:
+    an index far outside the configuration table.  So the pass over narrow
+    levels ends before it decodes anything when an entry failed, as the pass
+    over wide levels skips such an entry."""
+    a, b = 10, 6
+    i = j = (0 - 1) & 0xFFFFFFFF
+    assert (i * b + j) & 0xFFFFFFFF >= a * b
+    text = source("mc_pe_ordered.cuh")
+    narrow = between(text, "if (blockIdx.x == 0)", "while (!end)")
+    load, after = narrow.split("__syncthreads();", 1)
+    assert re.search(r"if \(!entry\(.*s_flags = kPeFlagError;", load)
+    assert re.search(r"if \(s_flags & kPeFlagError\) end = 1;", after)
+    for call in re.finditer(r"pe_slots<PT, SMALL>\(p, own", text):  # wide levels: behind the check
+        assert "if (entry(" in text[:call.start()].rsplit("if (s < Wl)", 1)[1]
