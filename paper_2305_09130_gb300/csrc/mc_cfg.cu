@@ -795,8 +795,11 @@ __device__ void warp_role(const CfgLaunch& A) {
       if (lane == 0 && err) set_error(Q.ctrl, (int)err);
     }
     // completion, as for a block unit: the warp that finishes the pass's
-    // last configuration combines the pass
+    // last configuration combines the pass.  Every lane added widths of its
+    // own and will read others': __syncwarp orders them before lane 0's fence,
+    // and lane 0's second fence before them (shuffles order no memory)
     uint32_t last = 0;
+    __syncwarp();
     if (lane == 0) {
       __threadfence();
       const uint32_t done = atomicAdd(&Q.ctrl->units_done, 1u) + 1;
@@ -805,6 +808,7 @@ __device__ void warp_role(const CfgLaunch& A) {
       if (last) __threadfence();
     }
     last = __shfl_sync(0xffffffffu, last, 0);
+    __syncwarp();
     if (last) {
       if (skip) {
         if (lane == 0) Q.ctrl->skipped = 1;

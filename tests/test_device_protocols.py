@@ -35,3 +35,17 @@ def test_narrow_levels_decode_only_entries_that_appeared():
     assert re.search(r"if \(s_flags & kPeFlagError\) end = 1;", after)
     for call in re.finditer(r"pe_slots<PT, SMALL>\(p, own", text):  # wide levels: behind the check
         assert "if (entry(" in text[:call.start()].rsplit("if (s < Wl)", 1)[1]
+
+
+def test_a_warps_widths_are_ordered_before_its_completion():
+    """Lanes of a warp add level widths one by one; lane 0 alone fences and
+    counts the unit as done, and the lanes of the warp that finishes a pass sum
+    the widths.  Shuffles and votes order no memory, so a __syncwarp stands
+    between the additions and lane 0's fence, and between lane 0's second fence
+    and the sums."""
+    role = between(source("mc_cfg.cu"), "__device__ void warp_role", "__global__")
+    before, rest = role.split("__threadfence();", 1)
+    assert "__syncwarp();" in before[before.index("explore_unit_warp"):]
+    assert before.rstrip().endswith("if (lane == 0) {")
+    counted, combine = rest.split("cfg_epilogue_warp", 1)
+    assert counted.index("units_done") < counted.index("__threadfence();") < counted.index("__syncwarp();")
