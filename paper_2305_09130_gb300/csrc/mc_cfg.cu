@@ -378,7 +378,9 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
   uint64_t vmin = kNone;
   while (L < 2 + N) {
     if (early && cut <= L) break;  // deeper widths are not counted
-    const uint32_t sc = early ? ld_relaxed_u32(&ctrl->stop_c) : 0u;
+    // (lane 0's: the word falls meanwhile and the lanes must leave together)
+    uint32_t sc = 0;
+    if (early && lane == 0) sc = ld_relaxed_u32(&ctrl->stop_c);
     const bool valid = my < W;
     C clk = 0;
     if (valid && unit_ok) clk = (C)field(key, c_shift, n_mask) * t_c;
@@ -400,7 +402,10 @@ __device__ uint32_t explore_unit_warp(const CfgPass& Q, uint32_t cfg, uint64_t T
     // the next level: state r from winner number r
     const uint32_t r = my < Wn ? my : 0u;
     key = shfl_key<K>(succ, Wn ? nth_set_bit(wm, r) : 0u);
-    cut = sc ? ~sc : kNoLevel;
+    if (early) {
+      sc = __shfl_sync(0xffffffffu, sc, 0);
+      cut = sc ? ~sc : kNoLevel;
+    }
     W = Wn;
     ++L;
     if (W == 0) break;

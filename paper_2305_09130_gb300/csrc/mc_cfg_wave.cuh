@@ -303,9 +303,13 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
   bool done = false;             // the terminal level was reached
   // early exit: the least level known to hold a violating terminal, asked
   // for at the end of a window and used at the next, so the load never holds
-  // a level up (a later stop only explores levels that are not counted)
-  uint32_t asked = early ? ld_relaxed_u32(&ctrl->stop_c) : 0u;
-  const bool beyond = k0 && asked && ~asked <= 2 + k0;  // below the first violating level: not counted
+  // a level up (a later stop only explores levels that are not counted).
+  // Other units lower the word meanwhile, and it decides which collectives
+  // the warp reaches: lane 0 reads it, and all lanes use its value.
+  uint32_t asked = 0;  // (lane 0's)
+  if (early && lane == 0) asked = ld_relaxed_u32(&ctrl->stop_c);
+  const uint32_t first_cut = __shfl_sync(0xffffffffu, asked, 0);
+  const bool beyond = k0 && first_cut && ~first_cut <= 2 + k0;  // below the first violating level: not counted
   while (reached && !beyond && sum < k1) {
     uint32_t late = 0;
     // waves of one unit, the common ones of uneven speeds: one state per
@@ -324,9 +328,9 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
       ones = 0;
       window = (before + 1) >> 5;
       if (early) {
-        const uint32_t cut = asked ? ~asked : 0xFFFFFFFFu;
-        if (cut <= before) break;  // deeper widths are not counted
-        asked = ld_relaxed_u32(&ctrl->stop_c);
+        const uint32_t known = __shfl_sync(0xffffffffu, asked, 0);
+        if (known && ~known <= before) break;  // deeper widths are not counted
+        if (lane == 0) asked = ld_relaxed_u32(&ctrl->stop_c);
       }
     }
     const uint32_t e = __popc(E);

@@ -49,3 +49,21 @@ def test_a_warps_widths_are_ordered_before_its_completion():
     assert before.rstrip().endswith("if (lane == 0) {")
     counted, combine = rest.split("cfg_epilogue_warp", 1)
     assert counted.index("units_done") < counted.index("__threadfence();") < counted.index("__syncwarp();")
+
+
+def test_the_first_violating_level_is_read_by_one_lane():
+    """The word with the least violating level falls while units run, and it
+    decides whether a warp goes on to its next shuffle or vote.  Were it read
+    by every lane, two lanes could see two values and part at a collective: one
+    lane reads it, and the value it saw is shuffled to all before it decides
+    anything."""
+    units = [between(source("mc_cfg_wave.cuh"), "__device__ void explore_unit_wave", "template <class K, class C>"),
+             between(source("mc_cfg.cu"), "__device__ uint32_t explore_unit_warp", "constexpr uint32_t kChainMaxP")]
+    for text in units:
+        reads = [m.start() for m in re.finditer(r"ld_relaxed_u32\(&ctrl->stop_c\)", text)]
+        assert reads
+        for at in reads:
+            line = text[text.rindex("\n", 0, at) + 1:at]
+            word = re.search(r"lane == 0\) (\w+) = $", line)
+            assert word, line
+            assert f"__shfl_sync(0xffffffffu, {word[1]}, 0)" in text
