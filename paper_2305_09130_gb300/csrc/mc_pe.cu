@@ -78,6 +78,7 @@ struct PeArgs {
   uint32_t slots;    // successors per lane: ceil(lanes / TILE) <= slots_for(TILE)
   uint32_t tag_bits; // ordered expansion: the log's tag (mc_explore.cuh), 0 bits: untagged
   uint64_t tag;
+  uint32_t solo_mask; // ordered expansion: block 0 meets the others when level & solo_mask is 0
 };
 
 struct Unit {
@@ -791,6 +792,7 @@ int pe_enqueue(mc_pe_model* m, uint64_t T, const uint64_t* T_src, int64_t delta,
   A.tmin_out = tmin_out;
   A.bar = m->d_bar;
   A.timeout_ns = m->opt.barrier_timeout_ns ? m->opt.barrier_timeout_ns : 60ull * 1000000000ull;
+  A.solo_mask = mc::pe_solo_mask(A.timeout_ns);
   const uint32_t lanes = m->P * m->M + m->P + 1;
   A.slots = (lanes + m->lay.tile - 1) / m->lay.tile;
   static_assert(sizeof(Ctrl) <= 256, "control block header");

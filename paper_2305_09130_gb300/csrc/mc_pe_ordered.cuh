@@ -27,8 +27,9 @@
 //
 // Levels of at most kPeSoloEnter states are explored by block 0 alone, the
 // frontier in shared memory and a block barrier per level, until one is wider
-// than kPeSoloCap; the other blocks wait at one device-wide barrier.  (Deep
-// programs run thousands of levels of a few dozen states.)  What bounds it:
+// than kPeSoloCap; the other blocks wait at a device-wide barrier, which block
+// 0 joins in time for their wait limit (pe_solo_mask).  (Deep programs run
+// thousands of levels of a few dozen states.)  What bounds it:
 // the chain of a level -- decode, reserve, poll -- not bytes or instructions
 // (a fifth of the issue slots are used).  Min-time queries of the abstract
 // kernel's model (39M states, 1,531 levels) 57.2 -> 21.0 ms against the pass
@@ -48,6 +49,20 @@ constexpr int kPeKeys = 2;               // states per thread and tile
 constexpr uint32_t kPeSoloCap = 1024;    // states of a level in shared memory
 constexpr uint32_t kPeSoloEnter = 512;
 constexpr uint32_t kPeSoloLine = 3;      // the barrier's spare line: how block 0's levels ended
+
+// Block 0 leaves the narrow levels at every level that is a multiple of a power
+// of two (and the other blocks come back with it), so that their wait stays
+// within the wait limit however many narrow levels there are: ten times what
+// one takes (2.4 us) for each.  One mask of the level, because the loop is a
+// chain that shows every instruction: with the clock read at the levels, or a
+// last level kept in a register, searches of the Minimum kernel's model took
+// 2 to 3% longer.
+constexpr uint64_t kPeSoloLevelNs = 24000;
+inline uint32_t pe_solo_mask(uint64_t timeout_ns) {
+  uint32_t every = 1;  // (levels stay below 2^30)
+  while (every < 1u << 30 && 2ull * every * kPeSoloLevelNs <= timeout_ns) every *= 2;
+  return every - 1;
+}
 
 struct PeSoloShared {
   u128 keys[2][kPeSoloCap];
@@ -378,7 +393,7 @@ __global__ void __launch_bounds__(kPeThreads, 2) pe_ordered_kernel(const __grid_
             n = done;
             cur ^= 1;
             if ((violated && A.early_exit) || L >= p.max_level) end = 1;
-            else if (n > kPeSoloCap) end = 2;  // back to every block
+            else if (n > kPeSoloCap || (L & A.solo_mask) == 0) end = 2;  // back to every block
           }
           __syncthreads();
           if (tid == 0) s_best = kNone;
