@@ -165,7 +165,10 @@ typedef struct {
                                    else 2^table_log2 slots                   */
   uint32_t threads_per_block;   /* 0: 256; else 64..256, multiple of 32      */
   uint32_t blocks_per_sm;       /* 0: occupancy maximum                      */
-  uint32_t max_probes;          /* 0: whole table; else bucket probe limit   */
+  uint32_t max_probes;          /* 0: whole table; else bucket probe limit.
+                                   Set on a FREE model that keeps no visited
+                                   set (mc_probe_scheme), it makes the next
+                                   query lay the buffers out again, with one */
   uint64_t log_capacity;        /* 0: closed-form bound; else states kept in
                                    the frontier log (MC_ERR_FRONTIER beyond) */
   uint64_t barrier_timeout_ns;  /* 0: 60 s.  Limit of each device-wide wait  */
@@ -320,7 +323,8 @@ void mc_model_destroy(mc_model* m);
 /* Replace the options of later queries.  Options that size buffers or the
  * launch (load_factor_pct, table_log2, log_capacity, threads_per_block,
  * blocks_per_sm, probe_scheme, no_log_tags, engine, unit_threads,
- * lanes_per_state) only act before the buffers exist.  Errors: INVAL. */
+ * lanes_per_state) only act before the buffers exist; max_probes acts on the
+ * next query (see there).  Errors: INVAL. */
 int mc_set_options(mc_model* m, const mc_options* opt);
 
 /* CUDA stream (a cudaStream_t, NULL = legacy default stream) for every later

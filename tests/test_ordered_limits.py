@@ -1,6 +1,7 @@
 """Ordered expansion of FREE models at the limits of its arithmetic: clocks
 that exceed 32 bits by a unit's speed alone, and keys that fill their word,
-compared with the oracle and with the pass that keeps a visited set."""
+compared with the oracle and with the pass that keeps a visited set; and a
+probe limit set on a model that keeps none so far."""
 import pytest
 
 import replay as RP
@@ -70,3 +71,27 @@ def test_keys_that_fill_their_word(mc):
         got.append({k: v for k, v in r.items() if k != "trace"})
         mc.mc_model_destroy(m)
     assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("allocator", ["torch", None])
+def test_a_probe_limit_set_later_acts(mc, allocator):
+    """mc_options.max_probes acts on later queries, also of a model that was
+    laid out without a visited set: one bucket probe cannot place the wide
+    levels of 737,855 states, 64 can."""
+    spec = W.c2(G=40, rule=W.FREE)
+    m = mc.mc_model_create(spec, mc.mc_options_default(engine="level"), allocator=allocator)
+    small = mc.mc_model_layout(m)["device_bytes"]
+    exp = mc.mc_min_time(m, trace=False)
+    assert mc.mc_count_states(m) == 737_855
+    widths = mc.mc_last_widths(m)
+    for limit in (1, 64, 1, 0):
+        mc.mc_set_options(m, mc.mc_options_default(engine="level", max_probes=limit))
+        if limit == 1:
+            with pytest.raises(mc.MCError) as e:
+                mc.mc_count_states(m)
+            assert e.value.code == mc.MC_ERR_TABLE_FULL
+            assert mc.mc_model_layout(m)["device_bytes"] > small
+            continue
+        assert mc.mc_count_states(m) == 737_855 and mc.mc_last_widths(m) == widths
+        assert mc.mc_min_time(m, trace=False) == exp
+    mc.mc_model_destroy(m)
