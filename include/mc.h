@@ -262,7 +262,9 @@ typedef struct {
                             at a level's barrier before writing its last
                             entries: 8 to 16 where the key leaves that many
                             spare (a 128-bit key is stored as two words of
-                            64 - log_tag_bits payload bits), else 0        */
+                            64 - log_tag_bits payload bits; of a FREE model
+                            without a visited set, one of at most 56 used
+                            bits in the low word alone), else 0            */
   uint32_t engine;       /* MC_ENGINE_LEVEL or MC_ENGINE_CONFIG (AUTO
                             resolved); with CONFIG, table_slots is the
                             shared-memory table of one block and the log

@@ -482,10 +482,12 @@ uint32_t resolve_engine(const mc_model* m) {
 
 // spare top bits per 64-bit word of a key that tag the frontier log (8 to
 // 16), or 0: a 128-bit key is stored as two words of 64 - t payload bits
+// (ordered expansion keeps narrow ones in the low word: mc_tree.h)
 uint32_t log_tag_bits(const mc_model* m) {
   if (m->opt.no_log_tags) return 0;
   const uint32_t spare = m->key_words == 1 ? 64 - m->used_bits : (128 - m->used_bits) / 2;
-  return spare >= 8 ? std::min<uint32_t>(spare, 16) : 0;
+  const uint32_t bits = spare >= 8 ? std::min<uint32_t>(spare, 16) : 0;
+  return m->ordered ? mc::tree_tag_bits((int)m->key_words, m->used_bits, bits) : bits;
 }
 
 // the probe scheme of the exploration kernel: AUTO follows the key width
@@ -713,7 +715,6 @@ int reserve(mc_model* m) {
   // tagged frontier log for 64-bit keys with 8 or more spare top bits: the
   // log starts cleared, so no entry of freed memory carries a tag
   m->tag_bits = cfg ? 0 : log_tag_bits(m);  // the configuration engine's log is read only after its pass
-  if (m->ordered) m->tag_bits = mc::tree_tag_bits((int)m->key_words, m->used_bits, m->tag_bits);
   m->tag = 0;
   if (m->tag_bits) MC_CUDA(m, cudaMemsetAsync(m->d_log_keys, 0, m->log_cap * key_bytes, m->stream));
 

@@ -1,0 +1,32 @@
+"""mc_layout says what the passes use (no device needed)."""
+import pytest
+
+from paper_2305_09130_gb300 import mc
+from paper_2305_09130_gb300 import workloads as W
+
+
+@pytest.fixture(scope="module")
+def lib():
+    return mc.load()
+
+
+def layout(spec, **kw):
+    return mc.mc_model_layout(mc.mc_model_create(spec, mc.mc_options_default(engine="level", **kw), allocator=None))
+
+
+@pytest.mark.parametrize("n,used,general,ordered", [(7, 26, 16, 16), (63, 50, 16, 14), (127, 58, 16, 16)])
+def test_log_tag_bits_of_narrow_128_bit_keys(lib, n, used, general, ordered):
+    """Ordered expansion keeps 128-bit keys of at most 56 used bits in the low
+    word, tag above it: 64 - used bits at most.  A pass that probes a visited
+    set, and keys of more used bits, spread the key over both words."""
+    spec = W.ModelSpec("narrow", 8, [1], [1], [n], [1], [1] * 8, key_bits=128)
+    assert layout(spec)["used_bits"] == used
+    assert layout(spec)["log_tag_bits"] == ordered
+    assert layout(spec, probe_scheme="split")["log_tag_bits"] == general
+    assert layout(spec.with_rule(W.GREEDY))["log_tag_bits"] == general
+    assert layout(spec, no_log_tags=1)["log_tag_bits"] == 0
+
+
+def test_log_tag_bits_of_c3_star(lib):
+    lay = layout(W.c3_star())
+    assert (lay["used_bits"], lay["log_tag_bits"]) == (55, 9)
