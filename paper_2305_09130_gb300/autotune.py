@@ -206,17 +206,17 @@ def tune_batch(specs, queries, space=None, reps: int = 2, cache: Optional[dict] 
     return {"signature": sig, **out}
 
 
-PE_SPACE = {
-    "lanes_per_state": [8, 16, 32],
-    "blocks_per_sm": [0, 1, 2],
-}
+# (no lanes_per_state: the ordered pass takes a thread per state whatever it
+# says, so candidates that differ in it alone would be told apart by noise)
+PE_SPACE = {"blocks_per_sm": [0, 1, 2]}
 
 
 def tune_pe(spec, query: str = "min_time", space=None, reps: int = 2, cache: Optional[dict] = None,
             path: Optional[str] = None) -> dict:
-    """Tune the PE-level model's query ("count" or "min_time"): lanes per
-    state (the warp tile that expands one state) and the persistent grid.
-    Candidates whose tile cannot hold the model's successors are skipped."""
+    """Tune the PE-level model's query ("count" or "min_time"): the persistent
+    grid.  A ``space`` of the pass with a visited set (``max_probes``) can name
+    ``lanes_per_state`` (the warp tile that expands one state) too; tiles that
+    cannot hold the model's successors are skipped."""
     from . import mc
 
     mc.load()

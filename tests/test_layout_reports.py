@@ -1,6 +1,8 @@
-"""mc_layout says what the passes use (no device needed)."""
+"""mc_layout says what the passes use, and the tuner's candidates differ in
+what they read (no device needed)."""
 import pytest
 
+from paper_2305_09130_gb300 import autotune as AT
 from paper_2305_09130_gb300 import mc
 from paper_2305_09130_gb300 import workloads as W
 
@@ -30,3 +32,9 @@ def test_log_tag_bits_of_narrow_128_bit_keys(lib, n, used, general, ordered):
 def test_log_tag_bits_of_c3_star(lib):
     lay = layout(W.c3_star())
     assert (lay["used_bits"], lay["log_tag_bits"]) == (55, 9)
+
+
+def test_pe_candidates_differ_in_what_the_ordered_pass_reads():
+    assert set(AT.PE_SPACE) == {"blocks_per_sm"}
+    cands = AT.candidates(AT.PE_SPACE)
+    assert len({c["blocks_per_sm"] for c in cands}) == len(cands) == 3
