@@ -251,7 +251,10 @@ typedef struct {
   uint64_t table_slots;  /* visited-set slots (what a named insert takes;
                             AUTO on a FREE model keeps no visited set, and
                             device_bytes leaves it out)                    */
-  uint64_t log_capacity; /* frontier-log entries                           */
+  uint64_t log_capacity; /* frontier-log entries (CONFIG: where blocks
+                            explore the configurations of a GREEDY model;
+                            other units keep no log, and device_bytes leaves
+                            it out)                                        */
   uint64_t max_width;    /* bound on one level's width                     */
   uint64_t state_bound;  /* bound on all reachable states (saturates)      */
   uint64_t device_bytes; /* device memory the model needs                  */

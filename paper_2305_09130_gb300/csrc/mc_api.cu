@@ -239,6 +239,7 @@ struct mc_model {
   int cfg_unit_threads = 0;  // mc_layout.unit_threads
   uint32_t cfg_segment = 0;  // wave units: work-groups of a segment (0: no wave units)
   uint64_t cfg_units = 0;    // units of a pass: configurations, or their segments
+  uint64_t cfg_log = 0;      // log entries its units keep: log_cap, or none
   // device state
   bool reserved = false;
   int device = -1;
@@ -516,7 +517,8 @@ int size_buffers(mc_model* m) {
   m->ordered = m->engine == MC_ENGINE_LEVEL && resolve_ordered(m);
   if (m->engine == MC_ENGINE_CONFIG) {
     if (!cfg_eligible(m)) return MC_ERR_INVAL;
-    // a segment of the log per configuration, shared-memory tables per block
+    // a segment of the log per configuration (where units keep one: below),
+    // shared-memory tables per block
     const uint64_t ab = (uint64_t)m->a * m->b;
     m->log_cap = m->unit_log;
     uint32_t w = 32;
@@ -542,6 +544,7 @@ int size_buffers(mc_model* m) {
     // subsets fit it (wave units), whatever its lanes per state
     m->cfg_warp = fits_warp || mc::wave_model(m->rule, m->P, m->opt.unit_threads);
     m->cfg_threads = m->cfg_warp ? (int)mc::kCfgWarpBlockThreads : m->cfg_unit_threads;
+    m->cfg_log = mc::cfg_keeps_log(m->rule, m->cfg_warp) ? m->log_cap : 0;
     m->cfg_segment = 0;
     m->cfg_units = ab;
     if (mc::wave_model(m->rule, m->P, m->opt.unit_threads)) {
@@ -553,7 +556,7 @@ int size_buffers(mc_model* m) {
     }
     const uint64_t key_bytes = 8ull * m->key_words;
     const uint64_t ctrl_bytes = (mc::kBarBytes + sizeof(Ctrl)) * kSlots + kScalarBytes + 8ull * (m->max_level + 2) * 5;
-    uint64_t total = mul_sat(m->log_cap, key_bytes + 4);
+    uint64_t total = mul_sat(m->cfg_log, key_bytes + 4);
     total = add_sat(total, ctrl_bytes + 4ull * (2 * ab + m->P));
     total = add_sat(total, 8 * (ab + 1) + 2 * sizeof(mc::CfgRec) * ab + 28 * m->cfg_units + 8 * sizeof(mc::CfgPass));
     total = add_sat(total, 16ull * (m->max_level + 2) * kSlots);  // level widths per result slot
@@ -680,8 +683,9 @@ int reserve(mc_model* m) {
   m->d_params = (uint32_t*)dev_alloc(m, np * 4);
   const bool table = !cfg && !m->ordered;
   if (table) m->d_table = dev_alloc(m, m->table_slots * key_bytes);
-  m->d_log_keys = dev_alloc(m, m->log_cap * key_bytes);
-  m->d_log_par = (uint32_t*)dev_alloc(m, m->log_cap * 4);
+  const uint64_t log_entries = cfg ? m->cfg_log : m->log_cap;
+  m->d_log_keys = dev_alloc(m, log_entries * key_bytes);
+  m->d_log_par = (uint32_t*)dev_alloc(m, log_entries * 4);
   const size_t L2 = m->max_level + 2;
   const size_t mirror_bytes = sizeof(Ctrl) * kSlots + kScalarBytes + 16 * L2;  // headers, scalars, trace
   const size_t ctrl_bytes = mc::kBarBytes * kSlots + mirror_bytes + 16 * L2 + 8 * L2;

@@ -92,7 +92,9 @@ int cfg_prepare(const mc_model_desc& d_in, const mc_options& o, CfgModelPrep& M,
   uint32_t w = 32;
   while (w < M.unit_width) w <<= 1;
   M.wcap = w;
-  // region: [params][seg][rec x 3][levels x 3][trace][log keys][log parents]
+  // region: [params][seg][rec x 3][levels x 3][trace], and where its units
+  // keep a log [log keys][log parents]
+  if (!cfg_keeps_log(M.p.rule, cfg_warp_model(M, o))) M.unit_log = 0;
   M.region = al256(4ull * M.params.size()) + al256(8ull * (M.ab + 1)) + al256(3ull * sizeof(CfgRec) * M.ab) +
              al256(48ull * M.L2) + al256(16ull * M.L2) + al256(16 * M.unit_log) + al256(4 * M.unit_log);
   return MC_OK;

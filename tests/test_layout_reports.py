@@ -1,5 +1,5 @@
-"""mc_layout says what the passes use, and the tuner's candidates differ in
-what they read (no device needed)."""
+"""mc_layout says what the passes use, memory is set aside for what they use,
+and the tuner's candidates differ in what they read (no device needed)."""
 import pytest
 
 from paper_2305_09130_gb300 import autotune as AT
@@ -38,3 +38,22 @@ def test_pe_candidates_differ_in_what_the_ordered_pass_reads():
     assert set(AT.PE_SPACE) == {"blocks_per_sm"}
     cands = AT.candidates(AT.PE_SPACE)
     assert len({c["blocks_per_sm"] for c in cands}) == len(cands) == 3
+
+
+@pytest.mark.parametrize("spec,opts,keeps", [(W.c3(), {}, False), (W.c3(), {"unit_threads": 128}, True),
+                                             (W.c2(), {}, False), (W.c1(W.FREE), {}, False),
+                                             (W.c1(W.FREE), {"unit_threads": 64}, False),
+                                             (W.random_small(91, 11, 2, 2, 30, rule=W.GREEDY), {}, True)],
+                         ids=lambda x: getattr(x, "name", None) or str(x))
+def test_log_memory_only_where_units_keep_a_log(lib, spec, opts, keeps):
+    """Configuration engine: block units of GREEDY models keep a frontier log;
+    warps and FREE units do not, and nothing is set aside for one."""
+    o = mc.mc_options_default(engine="config", **opts)
+    spec = spec.with_key_bits(128)
+    lay = mc.mc_model_layout(mc.mc_model_create(spec, o, allocator=None))
+    log = 20 * lay["log_capacity"]
+    assert log > 0 and (lay["device_bytes"] > log) == keeps
+    batch = mc.mc_batch_create([spec], o, allocator=None)
+    size = mc.mc_batch_device_bytes(batch)
+    mc.mc_batch_destroy(batch)
+    assert (size > log) == keeps
