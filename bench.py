@@ -262,6 +262,22 @@ def ncu_traffic_per_launch(path: str, load_factor_pct: int, probe_scheme: str, s
 
 
 # ---------------------------------------------------------------- arms
+def config_units(spec, layout, opts):
+    """What explores a configuration on the configuration engine (kernel and
+    units), and whether it keeps a frontier log.  mc_layout.unit_threads holds
+    the threads of a configuration's widest level, which GREEDY models of up to
+    ten units do not need: warps explore them as waves."""
+    u = f"u{64 * layout['key_words']}"
+    if spec.rule == W.GREEDY and spec.P <= 10 and not opts.unit_threads:
+        return f"cfg_warp_kernel<{u}> (wave units: a warp per configuration, or per segment of a deep one)", False
+    if layout["unit_threads"] == 32:
+        return f"cfg_warp_kernel<{u}> (a warp per configuration)", False
+    threads = f"{layout['unit_threads']} threads per configuration"
+    if spec.rule == W.FREE and 2 <= spec.P <= 4:
+        return f"cfg_kernel<{u}> (chain units, {threads})", False
+    return f"cfg_kernel<{u}> ({threads})", spec.rule == W.GREEDY
+
+
 def cpu_baseline_sample(spec, wl: Workload, t_min: int) -> dict:
     """The oracle as it stands on a bounded sample of the workload: a pruned
     check(T) (the states of time <= T) or, for a workload the oracle finishes
@@ -461,8 +477,7 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
                           (f"explore_kernel<u{64 * layout['key_words']}, tile {1 << (spec.P - 1).bit_length()}, "
                            f"{'FREE' if spec.rule == W.FREE else 'GREEDY'}, {scheme} insert>"
                            if layout["engine"] == mc.ENGINE["level"] else
-                           f"cfg_kernel<u{64 * layout['key_words']}> ({layout['unit_threads']} threads per "
-                           f"configuration)"),
+                           config_units(spec, layout, opts)[0]),
                 "peak_source": f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"
                                if peak_kind == "measured" else "fallback 6.8 TB/s",
                 "launch_timing": "CUDA events on the model's stream, one pair around each query's chained "
@@ -573,7 +588,9 @@ def measure_single(args, name: str, steps: int, warmup: int, device, stream, loc
                    "probe_scheme": scheme,
                    "load_factor_pct": layout_lf(opts),
                    "visited_set_bytes": 0 if ordered else layout["table_slots"] * 8 * layout["key_words"],
-                   "frontier_log_bytes": layout["log_capacity"] * (8 * layout["key_words"] + 4),
+                   "frontier_log_bytes": (layout["log_capacity"] * (8 * layout["key_words"] + 4)
+                                          if layout["engine"] == mc.ENGINE["level"] or
+                                          config_units(spec, layout, opts)[1] else 0),
                    "states_per_step": states_local / steps,
                    "checks_per_step": r["checks"]},
         "time_to_optimal_config_ms": dev_ms_max / steps,

@@ -2,6 +2,7 @@
 and the tuner's candidates differ in what they read (no device needed)."""
 import pytest
 
+import bench
 from paper_2305_09130_gb300 import autotune as AT
 from paper_2305_09130_gb300 import mc
 from paper_2305_09130_gb300 import workloads as W
@@ -57,3 +58,16 @@ def test_log_memory_only_where_units_keep_a_log(lib, spec, opts, keeps):
     size = mc.mc_batch_device_bytes(batch)
     mc.mc_batch_destroy(batch)
     assert (size > log) == keeps
+    assert bench.config_units(spec, lay, o)[1] == keeps
+
+
+def test_bench_names_what_explores_a_configuration(lib):
+    def units(spec, **kw):
+        o = mc.mc_options_default(engine="config", **kw)
+        return bench.config_units(spec, mc.mc_model_layout(mc.mc_model_create(spec, o, allocator=None)), o)[0]
+
+    assert "wave units" in units(W.c3()) and "wave units" in units(W.c2()) and "u128" in units(W.c3())
+    assert units(W.c3(), unit_threads=128) == "cfg_kernel<u128> (128 threads per configuration)"
+    assert units(W.c1(W.FREE)) == "cfg_kernel<u64> (chain units, 256 threads per configuration)"
+    assert units(W.random_small(92, 1, 2, 2, 9)) == "cfg_warp_kernel<u64> (a warp per configuration)"
+    assert "threads per configuration" in units(W.random_small(91, 11, 2, 2, 30, rule=W.GREEDY))
