@@ -1927,10 +1927,13 @@ int mc_server_submit(mc_server* S, const mc_model_desc* desc, const mc_query* q,
   int rc = MC_ERR_INVAL;
   if (S->opt.engine != MC_ENGINE_LEVEL) {
     // the configuration engine when it takes the model and it fits a job
-    // A server without pruning keeps the block units for levels wider than a
-    // warp: its exhaustive searches are the long requests that others are
-    // seen to join and overtake (C3 literal outlasts 2 ms on blocks, not as
-    // waves); with pruning, the default, wave units answer every request.
+    // Without pruning, GREEDY levels wider than a warp keep the block units,
+    // which are slower (a min-time request on C3 literal 9.1 ms against 0.78 as
+    // waves, on C2 literal, whose levels fit a warp and take waves, 0.35): the
+    // overlap test of the request loop (test_requests_join_while_others_run)
+    // needs such a search to last longer than the 2 ms after which it submits
+    // the requests that overtake it.  With pruning, the default, every request
+    // takes waves.
     rc = mc::cfg_prepare(*desc, S->opt, req.cm, S->opt.prune != 0, false);
     if (rc == MC_OK && (req.cm.ab > kJobUnits || mc::cfg_tables_bytes(req.cm) > kJobTables)) rc = MC_ERR_INVAL;
     if (rc == MC_OK) {
