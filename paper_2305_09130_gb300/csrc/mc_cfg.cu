@@ -715,27 +715,49 @@ __device__ void cfg_epilogue_warp(const CfgPass& Q, uint64_t T) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t ab = p.a * p.b;
   if (ld_relaxed_u32(&Q.ctrl->err)) return;
+  // (loads first, eight configurations a lane in flight: this warp alone goes
+  // through all of them, about 100 us less for 62,500 that violate)
+  constexpr uint32_t kAhead = 8;
+  const uint32_t deep_seg = wave_unit(p) ? ld_relaxed_u32(&Q.ctrl->pad1[0]) : 0u;  // (segments': their records leave it out)
   uint64_t best = kNone;
   uint32_t stop = kNoLevel, deep = 2;
-  for (uint32_t cfg = lane; cfg < ab; cfg += 32) {
-    const uint64_t v = __ldcg(&Q.rec[cfg].vpack);
-    const uint32_t d = __ldcg(&Q.rec[cfg].deepest);
-    deep = d > deep ? d : deep;
-    if (v != kNone) {
-      const uint32_t s = 2u + __ldg(p.N + cfg);
-      stop = s < stop ? s : stop;
-      best = v < best ? v : best;
+  for (uint32_t c0 = lane; c0 < ab; c0 += 32 * kAhead) {
+    uint64_t v[kAhead];
+    uint32_t d[kAhead], n[kAhead];
+#pragma unroll
+    for (uint32_t k = 0; k < kAhead; ++k) {
+      const uint32_t cfg = c0 + 32 * k;
+      const bool in = cfg < ab;
+      v[k] = in ? __ldcg(&Q.rec[cfg].vpack) : kNone;
+      d[k] = in ? __ldcg(&Q.rec[cfg].deepest) : 0u;
+      n[k] = in ? __ldg(p.N + cfg) : 0u;
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < kAhead; ++k) {
+      deep = d[k] > deep ? d[k] : deep;
+      if (v[k] == kNone) continue;
+      stop = 2u + n[k] < stop ? 2u + n[k] : stop;
+      best = v[k] < best ? v[k] : best;
     }
   }
-  if (wave_unit(p)) deep = max(deep, ld_relaxed_u32(&Q.ctrl->pad1[0]));  // (wave units' records leave it out)
+  deep = max(deep, deep_seg);
   deep = __reduce_max_sync(0xffffffffu, deep);
   stop = __reduce_min_sync(0xffffffffu, stop);
   best = warp_min_u64(best);
   uint64_t wpack = kNone;
   if (stop != kNoLevel) {
-    for (uint32_t cfg = lane; cfg < ab; cfg += 32) {
-      const uint64_t v = __ldcg(&Q.rec[cfg].vpack);
-      if (v != kNone && 2u + __ldg(p.N + cfg) == stop) wpack = v < wpack ? v : wpack;
+    for (uint32_t c0 = lane; c0 < ab; c0 += 32 * kAhead) {
+      uint64_t v[kAhead];
+      uint32_t n[kAhead];
+#pragma unroll
+      for (uint32_t k = 0; k < kAhead; ++k) {
+        const uint32_t cfg = c0 + 32 * k;
+        v[k] = cfg < ab ? __ldcg(&Q.rec[cfg].vpack) : kNone;
+        n[k] = cfg < ab ? __ldg(p.N + cfg) : 0u;
+      }
+#pragma unroll
+      for (uint32_t k = 0; k < kAhead; ++k)
+        if (2u + n[k] == stop && v[k] < wpack) wpack = v[k];
     }
     wpack = warp_min_u64(wpack);
   }
@@ -764,40 +786,59 @@ __device__ void cfg_epilogue_warp(const CfgPass& Q, uint64_t T) {
 template <class K>
 __device__ void warp_role(const CfgLaunch& A) {
   const uint32_t lane = threadIdx.x & 31u;
-  for (;;) {
-    uint32_t u = 0;
-    if (lane == 0) u = atomicAdd(A.wnext, 1u);
-    u = __shfl_sync(0xffffffffu, u, 0);
-    const uint64_t n = A.n_wunits_dev ? (uint64_t)*A.n_wunits_dev : A.n_wunits;
-    if (u >= n) return;
-    const uint64_t code = A.wunits ? __ldg(A.wunits_rev ? A.wunits - u : A.wunits + u) : 0ull;
-    const CfgPass& Q = A.wunits ? A.passes[code >> 32] : A.one;
-    // a configuration, or (wave units: Q.group holds the segments' length
-    // above the lanes per state) a segment of one
-    const uint32_t part = A.wunits ? (uint32_t)code : __ldg(Q.order + u);
-    const uint32_t segment = Q.group >> 8;
-    const uint32_t cfg = segment ? part & 0xFFFFFFu : part;
-    // the threshold, as for a block unit
-    unsigned long long t = 0;
-    uint32_t skip = 0;
-    if (lane == 0) {
-      t = Q.T;
-      if (Q.T_src) t = ld_relaxed_u64(Q.T_src) + (uint64_t)Q.T_delta;
-      if (Q.prev) {
-        const Ctrl* q = Q.prev;
-        if (ld_relaxed_u32(&q->err) || ld_relaxed_u32(&q->skipped) || ld_relaxed_u32(&q->stop_level) == 0) skip = 1;
-        else t = pack_time(ld_relaxed_u64(&q->wpack)) - 1;
-      }
+  const uint64_t n = A.n_wunits_dev ? (uint64_t)*A.n_wunits_dev : A.n_wunits;
+  // A launch of one pass with a warp for every unit: each takes its own,
+  // without a counter (a round trip less of a short pass's chain: 12.0 -> 10.4
+  // us for 256 configurations).  With more units a warp counts those it
+  // finished and adds them when none is left: atomics on one word bound passes
+  // of many small configurations, and this halves them (62,500: 425 -> 363 us).
+  // Launches of many passes share the device with others, so their units go to
+  // the warps that run, one at a time.
+  const bool one_each = !A.wunits && (uint64_t)A.warp_blocks * (blockDim.x >> 5) >= n;
+  uint32_t finished = 0;  // (units not yet added to units_done)
+  unsigned long long t = 0;
+  uint32_t skip = 0;
+  for (bool more = true; more;) {
+    uint32_t u = (threadIdx.x >> 5) * A.warp_blocks + blockIdx.x;
+    if (!one_each) {
+      if (lane == 0) u = atomicAdd(A.wnext, 1u);
+      u = __shfl_sync(0xffffffffu, u, 0);
     }
-    t = __shfl_sync(0xffffffffu, t, 0);
-    skip = __shfl_sync(0xffffffffu, skip, 0);
-    if (!skip && wave_unit(Q.p)) {
-      if (Q.p.clk32) explore_wave<K, uint32_t>(Q, cfg, t, segment, segment ? part >> 24 : 0u);
-      else explore_wave<K, uint64_t>(Q, cfg, t, segment, segment ? part >> 24 : 0u);
-    } else if (!skip) {
-      const uint32_t err = Q.p.clk32 ? explore_unit_warp<K, uint32_t>(Q, cfg, t)
-                                     : explore_unit_warp<K, uint64_t>(Q, cfg, t);
-      if (lane == 0 && err) set_error(Q.ctrl, (int)err);
+    more = u < n && !one_each;
+    if (u >= n && !finished) return;
+    const bool unit = u < n;
+    const uint64_t code = A.wunits ? __ldg(A.wunits_rev ? A.wunits - u : A.wunits + u) : 0ull;  // (unit: finished is 0 here)
+    const CfgPass& Q = A.wunits ? A.passes[code >> 32] : A.one;
+    const uint32_t segment = Q.group >> 8;
+    if (unit) {
+      // a configuration, or (wave units: Q.group holds the segments' length
+      // above the lanes per state) a segment of one
+      const uint32_t part = A.wunits ? (uint32_t)code : __ldg(Q.order + u);
+      const uint32_t cfg = segment ? part & 0xFFFFFFu : part;
+      // the threshold, as for a block unit
+      t = 0;
+      skip = 0;
+      if (lane == 0) {
+        t = Q.T;
+        if (Q.T_src) t = ld_relaxed_u64(Q.T_src) + (uint64_t)Q.T_delta;
+        if (Q.prev) {
+          const Ctrl* q = Q.prev;
+          if (ld_relaxed_u32(&q->err) || ld_relaxed_u32(&q->skipped) || ld_relaxed_u32(&q->stop_level) == 0) skip = 1;
+          else t = pack_time(ld_relaxed_u64(&q->wpack)) - 1;
+        }
+      }
+      t = __shfl_sync(0xffffffffu, t, 0);
+      skip = __shfl_sync(0xffffffffu, skip, 0);
+      if (!skip && wave_unit(Q.p)) {
+        if (Q.p.clk32) explore_wave<K, uint32_t>(Q, cfg, t, segment, segment ? part >> 24 : 0u);
+        else explore_wave<K, uint64_t>(Q, cfg, t, segment, segment ? part >> 24 : 0u);
+      } else if (!skip) {
+        const uint32_t err = Q.p.clk32 ? explore_unit_warp<K, uint32_t>(Q, cfg, t)
+                                       : explore_unit_warp<K, uint64_t>(Q, cfg, t);
+        if (lane == 0 && err) set_error(Q.ctrl, (int)err);
+      }
+      ++finished;
+      if (!A.wunits && more) continue;
     }
     // completion, as for a block unit: the warp that finishes the pass's
     // last configuration combines the pass.  Every lane added widths of its
@@ -807,11 +848,12 @@ __device__ void warp_role(const CfgLaunch& A) {
     __syncwarp();
     if (lane == 0) {
       __threadfence();
-      const uint32_t done = atomicAdd(&Q.ctrl->units_done, 1u) + 1;
+      const uint32_t done = atomicAdd(&Q.ctrl->units_done, finished) + finished;
       const uint32_t ab = Q.p.a * Q.p.b;
       last = done == (segment ? (uint32_t)__ldg(Q.seg) : ab);  // (wave units keep no log: their number)
       if (last) __threadfence();
     }
+    finished = 0;
     last = __shfl_sync(0xffffffffu, last, 0);
     __syncwarp();
     if (last) {

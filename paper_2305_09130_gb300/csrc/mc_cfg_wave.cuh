@@ -270,10 +270,8 @@ struct WaveClocks<C, 0> {
 };
 
 // The positions (see above) of the units `mask`, a subset of E.
-__device__ __forceinline__ uint32_t wave_positions(uint32_t E, uint32_t mask) {
-  uint32_t A = 0;
-  for (uint32_t rest = mask; rest; rest &= rest - 1) A |= 1u << (__popc(E >> (__ffs(rest) - 1)) - 1);
-  return A;
+__device__ __forceinline__ uint32_t wave_positions(uint32_t E, uint32_t mask, uint32_t lane) {
+  return __reduce_or_sync(0xffffffffu, (mask >> lane) & 1u ? 1u << (__popc(E >> lane) - 1) : 0u);
 }
 
 // Explore work-groups k0 + 1 .. k1 of configuration `cfg` of pass Q at
@@ -308,8 +306,11 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
   // the warp reaches: lane 0 reads it, and all lanes use its value.
   uint32_t asked = 0;  // (lane 0's)
   if (early && lane == 0) asked = ld_relaxed_u32(&ctrl->stop_c);
-  const uint32_t first_cut = __shfl_sync(0xffffffffu, asked, 0);
-  const bool beyond = k0 && first_cut && ~first_cut <= 2 + k0;  // below the first violating level: not counted
+  bool beyond = false;  // a segment below the first violating level: not counted
+  if (k0) {
+    const uint32_t cut = __shfl_sync(0xffffffffu, asked, 0);
+    beyond = cut && ~cut <= 2 + k0;
+  }
   while (reached && !beyond && sum < k1) {
     uint32_t late = 0;
     // waves of one unit, the common ones of uneven speeds: one state per
@@ -354,7 +355,7 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
       sum += e;
       clocks.advance();
     } else {  // the last wave: the work-groups run out, or pruning keeps a unit from starting
-      const uint32_t A = wave_positions(E, E & ~late);
+      const uint32_t A = wave_positions(E, E & ~late, lane);
       const uint32_t m = min(N - sum, (uint32_t)__popc(A));
       cur = wave_part(A, m, lane, levels + 2ull * (before + 1), k0 > sum ? k0 - sum : 0u, k1 - sum);
       sum += m;
@@ -376,15 +377,15 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
     for (uint32_t rest = E; rest; rest &= rest - 1) {
       const C f = clocks.next(__ffs(rest) - 1);
       const C v = f > base_mx ? f : base_mx;
-      const uint32_t A = wave_positions(E, clocks.within(E, v));
-      if ((!hit || v < tv) && __any_sync(0xffffffffu, wave_within(cur, A, lane) != 0)) {
+      if (hit && v >= tv) continue;  // (units of one speed: the same time)
+      if (__any_sync(0xffffffffu, wave_within(cur, wave_positions(E, clocks.within(E, v), lane), lane) != 0)) {
         hit = true;
         tv = v;
       }
     }
     hit = hit && (uint64_t)tv <= T;
     if (hit) {
-      const uint32_t word = wave_within(cur, wave_positions(E, clocks.within(E, tv)), lane);
+      const uint32_t word = wave_within(cur, wave_positions(E, clocks.within(E, tv), lane), lane);
       const uint32_t who = __ffs(__ballot_sync(0xffffffffu, word != 0)) - 1;
       const uint32_t S = (who << 5) | (uint32_t)(__ffs(__shfl_sync(0xffffffffu, word, who)) - 1);
       key = ((K)(i + 1) << Q.p.wg_shift) | ((K)(j + 1) << Q.p.ts_shift);
@@ -394,8 +395,11 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
       }
     }
   }
-  // (pad1[0]: the deepest level any unit of the pass reached)
-  if (lane == 0 && reached) atomicMax(&ctrl->pad1[0], 2 + min(sum, k1));
+  // the deepest level reached: in the record, and by segments, which share one,
+  // in pad1[0] (one word for the pass: taken by every unit of 62,500
+  // configurations it lengthened a pass from 425 to 468 us)
+  const bool whole = k0 == 0 && k1 == N;
+  if (lane == 0 && reached && !whole) atomicMax(&ctrl->pad1[0], 2 + min(sum, k1));
   if (lane == 0 && k1 == N) {
     if (hit && early) atomicMax(&ctrl->stop_c, ~(2u + N));
     CfgRec rec;
@@ -403,7 +407,7 @@ __device__ void explore_unit_wave(const CfgPass& Q, uint32_t cfg, uint64_t T, ui
     rec.wkey_lo = hit ? KeyOps<K>::lo(key) : kNone;
     rec.wkey_hi = hit ? KeyOps<K>::hi(key) : kNone;
     rec.widx = 0;  // no log: wave_trace gives the path
-    rec.deepest = 0;
+    rec.deepest = whole ? 2 + sum : 0u;
     Q.rec[cfg] = rec;
   }
 }
