@@ -979,7 +979,11 @@ __global__ void cfg_clear_kernel(const CfgClear* clears, const uint32_t* n_dev) 
 
 // T_ini of every min-time model of a run: walk w of model k is random run
 // number w of its seed (as mc_simulate), the least terminal time wins.  A
-// warp per run.
+// warp per run, or a lane where the run's n models have enough of them.
+__device__ __forceinline__ bool sim_by_lanes(const CfgSim& s, uint32_t n) {
+  return (uint64_t)n * s.walks >= lane_runs(s.p.rule);
+}
+
 __global__ void cfg_sim_kernel(const CfgSim* sims, const uint32_t* n_dev, uint32_t walks_max) {
   const uint32_t n = *n_dev;
   const uint64_t total = (uint64_t)n * walks_max;
@@ -987,10 +991,28 @@ __global__ void cfg_sim_kernel(const CfgSim* sims, const uint32_t* n_dev, uint32
        x += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
     const uint32_t k = (uint32_t)(x / walks_max), w = (uint32_t)(x % walks_max);
     const CfgSim& s = sims[k];
-    if (w >= s.walks) continue;
+    if (w >= s.walks || sim_by_lanes(s, n)) continue;
     const uint64_t t = warp_walk_time(s.p, s.seed, w);
     if ((threadIdx.x & 31u) == 0)
       atomicMin(reinterpret_cast<unsigned long long*>(s.tini), (unsigned long long)t);
+  }
+}
+
+// The runs that take a lane each: a warp takes per_warp of a model's.
+__global__ void cfg_sim_runs_kernel(const CfgSim* sims, const uint32_t* n_dev, uint32_t walks_max, uint32_t per_warp) {
+  const uint32_t n = *n_dev, chunks = (walks_max + per_warp - 1) / per_warp;
+  for (uint64_t x = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < (uint64_t)n * chunks;
+       x += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
+    const CfgSim& s = sims[x / chunks];
+    const uint32_t first = (uint32_t)(x % chunks) * per_warp;
+    if (first >= s.walks || !sim_by_lanes(s, n)) continue;
+    const uint32_t runs = s.walks - first < per_warp ? s.walks - first : per_warp;
+    unsigned long long t;
+    if (!s.p.clk32) t = swarm_runs<uint64_t, 16>(s.p, s.seed, first, 0, runs, kNone);
+    else if (s.p.P <= 8) t = swarm_runs<uint32_t, 8>(s.p, s.seed, first, 0, runs, kNone);
+    else t = swarm_runs<uint32_t, 16>(s.p, s.seed, first, 0, runs, kNone);
+    t = warp_min_u64(t) >> 24;
+    if ((threadIdx.x & 31u) == 0) atomicMin(reinterpret_cast<unsigned long long*>(s.tini), t);
   }
 }
 
@@ -1006,6 +1028,11 @@ cudaError_t launch_cfg_clear(const CfgClear* clears, const uint32_t* n_dev, uint
 cudaError_t launch_cfg_sim(const CfgSim* sims, const uint32_t* n_dev, uint32_t n_max, uint32_t walks_max,
                            cudaStream_t stream) {
   if (n_max == 0 || walks_max == 0) return cudaSuccess;
+  if ((uint64_t)n_max * walks_max >= kLaneRunsGreedy) {  // (some models' runs may take a lane each)
+    const uint32_t per_warp = walks_max >= 256 ? 256 : (walks_max + 31) / 32 * 32;
+    const uint64_t all = ((uint64_t)n_max * ((walks_max + per_warp - 1) / per_warp) + 3) / 4;
+    cfg_sim_runs_kernel<<<(int)(all < 4096 ? all : 4096), 128, 0, stream>>>(sims, n_dev, walks_max, per_warp);
+  }
   const uint64_t blocks = ((uint64_t)n_max * walks_max + 3) / 4;  // 4 warps each
   const int grid = (int)(blocks < 4096 ? blocks : 4096);
   cfg_sim_kernel<<<grid, 128, 0, stream>>>(sims, n_dev, walks_max);

@@ -12,7 +12,7 @@ namespace {
 using namespace mc::dev;
 
 // ------------------------------------------------------------------ simulation (T_ini)
-// One random run per warp (Section 4, Step 3: a simulation gives T_ini).
+// Random runs (Section 4, Step 3: a simulation gives T_ini), one per warp.
 __global__ void simulate_kernel(const Params p, uint64_t seed, uint32_t walks, uint64_t* t_out) {
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -23,6 +23,17 @@ __global__ void simulate_kernel(const Params p, uint64_t seed, uint32_t walks, u
   }
   if ((threadIdx.x & 31u) == 0 && least != kNone)
     atomicMin(reinterpret_cast<unsigned long long*>(t_out), (unsigned long long)least);
+}
+
+// Many of them: a run per lane, as a swarm's (mc_walk.cuh), without a bound.
+template <class C, int PT>
+__global__ void simulate_runs_kernel(const Params p, uint64_t seed, uint32_t walks, uint32_t per_warp, uint64_t* t_out) {
+  const uint64_t first = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp;
+  if (first >= walks) return;
+  const uint32_t n = (uint32_t)(first + per_warp < walks ? per_warp : walks - first);
+  const unsigned long long mine = warp_min(swarm_runs<C, PT>(p, seed, first, 0, n, kNone));
+  if ((threadIdx.x & 31u) == 0 && mine != kNone)
+    atomicMin(reinterpret_cast<unsigned long long*>(t_out), mine >> 24);
 }
 
 // ------------------------------------------------------------------ swarm (Section 5)
@@ -165,9 +176,22 @@ cudaError_t launch_replay_walk(const Params& p, uint64_t seed, uint64_t w, int k
 cudaError_t launch_simulate(const Params& p, uint64_t seed, uint32_t walks, uint64_t* t_out,
                             cudaStream_t stream) {
   const int threads = 128;
-  const uint64_t blocks = ((uint64_t)walks * 32 + threads - 1) / threads;  // a warp per walk
-  const int grid = (int)(blocks < 4096 ? blocks : 4096);
-  simulate_kernel<<<grid, threads, 0, stream>>>(p, seed, walks, t_out);
+  if (walks < lane_runs(p.rule)) {
+    const uint64_t blocks = ((uint64_t)walks * 32 + threads - 1) / threads;
+    const int grid = (int)(blocks < 4096 ? blocks : 4096);
+    simulate_kernel<<<grid, threads, 0, stream>>>(p, seed, walks, t_out);
+    return cudaGetLastError();
+  }
+  uint32_t per_warp = 32;  // up to 4,096 warps
+  while ((uint64_t)per_warp * 4096 < walks) per_warp *= 2;
+  const uint32_t blocks = (uint32_t)(((uint64_t)walks + per_warp - 1) / per_warp + 3) / 4;  // 4 warps each
+#define MC_RUNS(PT)                                                                                          \
+  (p.clk32 ? simulate_runs_kernel<uint32_t, PT><<<blocks, threads, 0, stream>>>(p, seed, walks, per_warp, t_out) \
+           : simulate_runs_kernel<uint64_t, PT><<<blocks, threads, 0, stream>>>(p, seed, walks, per_warp, t_out))
+  if (p.P <= 4) MC_RUNS(4);
+  else if (p.P <= 8) MC_RUNS(8);
+  else MC_RUNS(16);
+#undef MC_RUNS
   return cudaGetLastError();
 }
 

@@ -20,14 +20,16 @@ namespace mc {
 namespace dev {
 
 // x % d for a divisor below 2^16 that stays the same: d's reciprocal (floor of
-// 2^32 / d) is multiplied instead of a 64-bit division's hundred instructions
-// (262,144 runs of C3 literal drew their configurations in three quarters of
-// the swarm's time).  A word's quotient comes out exact or one short, which
-// one conditional subtraction mends.
+// (2^32 - 1) / d) is multiplied instead of a 64-bit division's hundred
+// instructions (262,144 runs of C3 literal drew their configurations in three
+// quarters of the swarm's time).  A word's quotient comes out exact or one
+// short, which one conditional subtraction mends.
 struct FastMod {
   uint32_t d, inv, two32;  // two32 = 2^32 % d
-  __device__ explicit FastMod(uint32_t x)
-      : d(x), inv(x > 1 ? (uint32_t)(0x100000000ull / x) : 0xFFFFFFFFu), two32((uint32_t)(0x100000000ull % x)) {}
+  __device__ explicit FastMod(uint32_t x) : d(x), inv(0xFFFFFFFFu / x) {
+    const uint32_t rest = 0xFFFFFFFFu - inv * x + 1;
+    two32 = rest == x ? 0u : rest;
+  }
   __device__ __forceinline__ uint32_t word(uint32_t x) const {
     const uint32_t r = x - __umulhi(x, inv) * d;
     return r >= d ? r - d : r;
@@ -121,7 +123,7 @@ struct RunUnits {
     for (int c = 0; c < PT; ++c) {
       t[c] = c < (int)p.P ? (C)(cost * __ldg(p.speed + c)) : (C)1;
       clk[c] = 0;
-      if (sizeof(C) == 4) inv[c] = t[c] > 1 ? (uint32_t)(0x100000000ull / t[c]) : 0xFFFFFFFFu;
+      if (sizeof(C) == 4) inv[c] = 0xFFFFFFFFu / (uint32_t)t[c];
     }
   }
   __device__ __forceinline__ C over(C x, int c) const {  // x / t[c]
@@ -237,4 +239,16 @@ __device__ unsigned long long swarm_runs(const Params& p, uint64_t seed, uint64_
 }
 
 }  // namespace dev
+
+// Runs from which each takes a lane (swarm_runs) instead of a warp
+// (warp_walk_time).  A warp's 32 lanes share a run's draws (FREE) or its units
+// (GREEDY), which is faster while warps wait for work: 4,096 GREEDY runs of
+// 64-bit clocks take 58 us a warp each and 70 a lane each, 8,192 82 and 71;
+// 32,768 FREE runs of up to 400 work-groups 82 and 106, 131,072 218 and 205.
+// (16,384 runs of C1, GREEDY: 45 and 23 us; 1,048,576: 1,262 and 49, and 949
+// when a thread took a run step by step.)
+constexpr uint32_t kLaneRunsGreedy = 8192;
+constexpr uint32_t kLaneRunsFree = 131072;
+__host__ __device__ inline uint32_t lane_runs(uint32_t rule) { return rule == MC_GREEDY ? kLaneRunsGreedy : kLaneRunsFree; }
+
 }  // namespace mc
