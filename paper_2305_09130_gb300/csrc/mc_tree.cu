@@ -196,12 +196,19 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
     s_flags = 0;
     s_best = kNone;
   }
-  if (tid < kMaxP) {
-    uint32_t least = 0xFFFFFFFFu;
-    for (uint32_t f = 0; f < tid && f < p.P; ++f) least = min(least, __ldg(p.speed + p.P - 1 - f));
-    s_least[tid] = least;
+  if (warp == 0) {
+    const uint32_t own = lane < p.P ? __ldg(p.speed + p.P - 1 - lane) : 0u;
+    uint32_t least = __shfl_up_sync(0xffffffffu, own, 1);  // (lane 0's is not used)
+#pragma unroll
+    for (uint32_t o = 1; o < kMaxP; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, least, o);
+      if (lane > o) least = min(least, v);
+    }
+    if (lane < kMaxP) {
+      s_speed[lane] = own;
+      s_least[lane] = least;
+    }
   }
-  if (tid < kMaxP) s_speed[tid] = tid < p.P ? __ldg(p.speed + p.P - 1 - tid) : 0;
   // N_ij by the key's (i, j) bits, one lookup per state instead of two fields
   // and a gather; larger domains read the table in global memory
   const uint32_t ts_bits = p.wg_shift - p.ts_shift;
