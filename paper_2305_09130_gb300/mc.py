@@ -153,6 +153,10 @@ def _destroy_live_models():
         try:
             if isinstance(m, PeModel):
                 mc_pe_model_destroy(m)
+            elif isinstance(m, Batch):
+                mc_batch_destroy(m)
+            elif isinstance(m, Server):
+                mc_server_destroy(m)
             else:
                 mc_model_destroy(m)
         except Exception:
