@@ -36,6 +36,7 @@
 
 #include "mc_cfg_jobs.h"
 #include "mc_device.cuh"
+#include "mc_walk.h"
 
 namespace mc {
 namespace {
@@ -993,7 +994,7 @@ int batch_run_cfg(mc_batch* b, const mc_query* queries, mc_batch_result* results
   b->stats.h2d_bytes += b->run.upload_bytes;
   b->stats.d2h_bytes += b->run.result_bytes;
   b->stats.explore_launches += 2;
-  b->stats.other_launches += 2;
+  b->stats.other_launches += 2 + mc::sim_lanes_launch(b->run.cap_n, b->run.walks_max);
   if (b->opt.timing) {
     float ms = 0.f;
     MCB_CUDA(b, cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]));

@@ -1028,7 +1028,7 @@ cudaError_t launch_cfg_clear(const CfgClear* clears, const uint32_t* n_dev, uint
 cudaError_t launch_cfg_sim(const CfgSim* sims, const uint32_t* n_dev, uint32_t n_max, uint32_t walks_max,
                            cudaStream_t stream) {
   if (n_max == 0 || walks_max == 0) return cudaSuccess;
-  if ((uint64_t)n_max * walks_max >= kLaneRunsGreedy) {  // (some models' runs may take a lane each)
+  if (sim_lanes_launch(n_max, walks_max)) {
     const uint32_t per_warp = walks_max >= 256 ? 256 : (walks_max + 31) / 32 * 32;
     const uint64_t all = ((uint64_t)n_max * ((walks_max + per_warp - 1) / per_warp) + 3) / 4;
     cfg_sim_runs_kernel<<<(int)(all < 4096 ? all : 4096), 128, 0, stream>>>(sims, n_dev, walks_max, per_warp);

@@ -5,7 +5,7 @@
 // mode) in four launches on one stream, whatever the number of models:
 //   clear    every model's pass headers, level widths and {T_ini, T_min};
 //   sim      the T_ini simulation of every min-time model (Section 4,
-//            Step 3);
+//            Step 3; a fifth launch where the models have thousands of runs);
 //   pass A   every model's first pass: the min pass of a min-time query
 //            (pruned at T_ini, the least terminal time reduced on the
 //            device), or the check itself -- one unit per (model,

@@ -149,8 +149,8 @@ cudaError_t launch_swarm(const Params& p, uint64_t seed, uint64_t w0, uint32_t w
   // a warp takes 32 to 256 runs (several rounds of its lanes even long and
   // short runs out, but first every SM gets 16 warps), or as many as the
   // grid's warps need (`grid`: 8 blocks of 8 warps per SM).  A search of
-  // 262,144 runs a round on C3 literal takes 190 us with 256 runs to a warp
-  // and 129 us with 64.
+  // 262,144 runs a round on C3 literal took 190 us with 256 runs to a warp and
+  // 129 us with 64 (111 since its reciprocals take 32-bit divisions).
   const uint64_t warps = (uint64_t)grid * 8;
   uint32_t per_warp = 256;
   if ((uint64_t)per_warp * warps < walks) per_warp = (uint32_t)((walks + warps - 1) / warps);

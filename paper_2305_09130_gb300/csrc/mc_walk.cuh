@@ -15,6 +15,7 @@
 #include <cstdint>
 
 #include "mc_device.cuh"
+#include "mc_walk.h"
 
 namespace mc {
 namespace dev {
@@ -181,7 +182,7 @@ __device__ __forceinline__ C greedy_run(RunUnits<C, PT>& u, uint32_t P, uint32_t
 // warp's next run as soon as its own ends or passes the bound, so that lanes
 // do not wait for the longest of 32.  262,144 runs of C3 literal: 13.2 ms by
 // single steps with the clocks in local memory, 0.38 ms group by group (the
-// longest run's 512 groups in a row); the search of two rounds takes 0.19 ms
+// longest run's 512 groups in a row); the search of two rounds takes 0.11 ms
 // here, most of it launches and waits.
 template <class C, int PT>
 __device__ unsigned long long swarm_runs(const Params& p, uint64_t seed, uint64_t w0, uint32_t first, uint32_t last,
@@ -239,16 +240,4 @@ __device__ unsigned long long swarm_runs(const Params& p, uint64_t seed, uint64_
 }
 
 }  // namespace dev
-
-// Runs from which each takes a lane (swarm_runs) instead of a warp
-// (warp_walk_time).  A warp's 32 lanes share a run's draws (FREE) or its units
-// (GREEDY), which is faster while warps wait for work: 4,096 GREEDY runs of
-// 64-bit clocks take 58 us a warp each and 70 a lane each, 8,192 82 and 71;
-// 32,768 FREE runs of up to 400 work-groups 82 and 106, 131,072 218 and 205.
-// (16,384 runs of C1, GREEDY: 45 and 23 us; 1,048,576: 1,262 and 49, and 949
-// when a thread took a run step by step.)
-constexpr uint32_t kLaneRunsGreedy = 8192;
-constexpr uint32_t kLaneRunsFree = 131072;
-__host__ __device__ inline uint32_t lane_runs(uint32_t rule) { return rule == MC_GREEDY ? kLaneRunsGreedy : kLaneRunsFree; }
-
 }  // namespace mc
