@@ -163,7 +163,8 @@ typedef struct {
   uint32_t load_factor_pct;     /* visited-set load-factor cap, 10..90       */
   uint32_t table_log2;          /* 0: size the visited set from the bound;
                                    else 2^table_log2 slots                   */
-  uint32_t threads_per_block;   /* 0: 256; else 64..256, multiple of 32      */
+  uint32_t threads_per_block;   /* 0: 256 (PE-level model without a visited
+                                   set: 512); else 64..256, multiple of 32   */
   uint32_t blocks_per_sm;       /* 0: occupancy maximum                      */
   uint32_t max_probes;          /* 0: whole table; else bucket probe limit.
                                    Set on a FREE model that keeps no visited
@@ -186,7 +187,10 @@ typedef struct {
                                    from P (rounded up) to 16, one unit per
                                    lane; PE-level model (mc_pe.h): 4 or 8 (up
                                    to 3 successors per lane), 16 (up to 2) or
-                                   32 (1).  0 = the smallest that fits      */
+                                   32 (1).  0 = the smallest that fits.
+                                   Passes without a visited set (see
+                                   mc_probe_scheme, mc_pe.h) take a thread
+                                   per state whatever it says               */
   uint32_t probe_scheme;        /* mc_probe_scheme of the single-model
                                    explorer (mc_check, mc_min_time,
                                    mc_count_states); batches and the PE-level
