@@ -127,10 +127,10 @@ __device__ __forceinline__ bool tree_entry(const ExploreArgs& G, const TreeLog<K
 // terminal (FIN, Listing 4), those within T violate G(FIN -> time > T) (Step
 // 2), and the least of them lowers `best`.  The units of the fields below f0
 // have not started, so their next clocks are one work-group each; `least[f]`
-// (f > 0) is the least speed of the fields below f.  Clocks in C: 32 bits when
-// every clock of the model fits.  (One state in five has terminal successors
-// on C3 at G=36: with a loop per field and per successor in 64 bits this was
-// 40% of the pass.)
+// is the least speed of the fields below f (2^32 - 1 for f = 0).  Clocks in C:
+// 32 bits when every clock of the model fits.  (One state in five has terminal
+// successors on C3 at G=36: with a loop per field and per successor in 64 bits
+// this was 40% of the pass.)
 template <bool PRUNE, class C, class A>
 __device__ __forceinline__ void tree_times(const Params& p, A key, uint32_t f0, uint64_t cost, bool terminal,
                                            uint64_t T, uint32_t i, uint32_t j, const uint32_t* speed,
@@ -157,9 +157,10 @@ __device__ __forceinline__ void tree_times(const Params& p, A key, uint32_t f0, 
       if ((uint64_t)max(mx, (C)speed[f]) * cost > T) starts &= ~(1u << f);
   }
   if (terminal) {
-    // (no field below the lowest: only `own`, which 64-bit clocks may take
-    // beyond any 32-bit stand-in for "none")
-    const uint64_t t = (uint64_t)max(mx, f0 ? min(own, (C)least[f0]) : own) * cost;
+    // (no field below the lowest: least[0] is beyond every clock of 32 bits,
+    // but not of 64)
+    const C other = sizeof(C) == 8 && f0 == 0 ? (C)~(C)0 : (C)least[f0];
+    const uint64_t t = (uint64_t)max(mx, min(own, other)) * cost;
     if (t <= T && t <= pack_time(best)) best = min(best, pack_tij(t, i, j));
   }
 }
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
   }
   if (warp == 0) {
     const uint32_t own = lane < p.P ? __ldg(p.speed + p.P - 1 - lane) : 0u;
-    uint32_t least = __shfl_up_sync(0xffffffffu, own, 1);  // (lane 0's is not used)
+    uint32_t least = __shfl_up_sync(0xffffffffu, own, 1);
 #pragma unroll
     for (uint32_t o = 1; o < kMaxP; o <<= 1) {
       const uint32_t v = __shfl_up_sync(0xffffffffu, least, o);
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(kTreeThreads, 4) tree_kernel(const __grid_cons
     }
     if (lane < kMaxP) {
       s_speed[lane] = own;
-      s_least[lane] = least;
+      s_least[lane] = lane ? least : 0xFFFFFFFFu;
     }
   }
   // N_ij by the key's (i, j) bits, one lookup per state instead of two fields
