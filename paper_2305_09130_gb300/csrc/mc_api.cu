@@ -622,11 +622,11 @@ void fill_params(const mc_model* m, Params& p) {
 
 int reserve(mc_model* m) {
   m->chain_open = false;  // every query starts here; a run left open by a failed query is dropped
+  if (m->reserved && (!m->ordered || m->opt.max_probes == 0)) return MC_OK;
+  // max_probes acts on later queries, and a model laid out for ordered
+  // expansion has no visited set to probe: lay it out again, with one
   DeviceGuard guard(m->reserved ? m->device : -1);
   if (m->reserved) {
-    if (!m->ordered || m->opt.max_probes == 0) return MC_OK;
-    // max_probes acts on later queries, and a model laid out for ordered
-    // expansion has no visited set to probe: lay it out again, with one
     release(m);
     m->last_levels = 0;
   }
